@@ -436,9 +436,7 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
   k->prec = desc->precision;
   k->elem = (k->prec == BEM_FP64) ? sizeof(double) : sizeof(float);
   cudaGetDevice(&k->dev);
-  // radix 16 for every float pass until bem_set_radix or bem_autotune says otherwise
-  k->col_radix_alt = 0;
-  k->row_radix_alt = 0;
+  default_radix(k);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const size_t n = (size_t)k->N * k->N;
   Workspace& w = k->ws;

@@ -204,6 +204,16 @@ inline bool first_on_device(std::atomic<unsigned long long>& seen) {
   return (seen.fetch_or(bit) & bit) == 0;
 }
 
+// FFT radices of a new handle (bem_set_radix and bem_autotune change them).  Short float
+// transforms take radix 8: more threads and a shorter chain per thread on grids that do
+// not fill the GPU.  One product (GB300, radix 8 / 16): rows N = 256 7.2 / 7.4 us, 512
+// 13.0 / 10.4; columns N = 512 10.4 / 14.8, 1024 23.6 / 21.3.
+inline void default_radix(bem_kernel_s* k) {
+  const bool f32 = k->prec == BEM_FP32;
+  k->row_radix_alt = (f32 && k->logN <= 8) ? 1 : 0;
+  k->col_radix_alt = (f32 && k->logN <= 9) ? 1 : 0;
+}
+
 void set_error(const std::string& msg);
 // number of kernel launches issued by the library (for launch accounting)
 void note_launches(long long n);

@@ -20,13 +20,30 @@
 
 namespace bem {
 
-// Launch bounds per (precision, radix, pass): KIND 0 = rows, 1 = columns.
-template <typename T, int LOGR, int KIND> struct RegCfg { static constexpr int MAXT = 512, MINB = 2; };
-template <> struct RegCfg<float, 4, 1> { static constexpr int MAXT = 256, MINB = 3; };
-template <> struct RegCfg<float, 3, 0> { static constexpr int MAXT = 512, MINB = 3; };
-template <int KIND> struct RegCfg<double, 3, KIND> { static constexpr int MAXT = 512, MINB = 1; };
-template <int KIND> struct RegCfg<double, 4, KIND> { static constexpr int MAXT = 256, MINB = 1; };
-
+// Block shapes.  A block holds as few rows or columns as the memory accesses allow, so
+// that small and middle grids spread over all 152 SMs (one block of 512 threads per 16
+// to 64 rows had left N = 64 on one SM and N = 512 on 32), and large ones have many
+// small blocks whose waits interleave:
+//  - rows: two (float: their records of one frequency fill a 32-byte sector; double from
+//    N = 512, 156 / 169 us with one) or one (double, smaller grids);
+//  - columns: one pair of columns (float) or one column (double);
+//  - at least one warp per block.
+// Measured on GB300, one product inside a graph, 512-thread row blocks / 4 rows / 2 rows:
+// float N = 256: 9.0 / 7.4 / 7.2 us, 512: 14.2 / 10.7 / 10.4, 1024: 32.4 / 28.2 / 21.3,
+// 2048: - / 71.8 / 67.7; one row (half sectors): 1024: 32.6, 2048: 77.5.  Double, before
+// and now, N = 64: 128 / 29 us, 512: 160 / 156 us.
+// RES: the threads resident per SM that a pass's register budget is made for.  768 for
+// radix-16 rows (85 registers, nothing spilled) against 1024: N = 2048 67.7 / 69.2 us,
+// 1280: 78.5; the paired columns need 128 registers (512 threads; 768: 82 us).
+template <typename T, int LOGR, int KIND> struct RegCfg { static constexpr int RES = 768; };
+template <> struct RegCfg<float, 3, 0> { static constexpr int RES = 1536; };
+template <int KIND> struct RegCfg<double, 3, KIND> { static constexpr int RES = 512; };
+constexpr int kColPairRes = 512;
+__host__ __device__ constexpr int min_blocks(int threads, int res) {
+  return res / threads < 1 ? 1 : (res / threads > 24 ? 24 : res / threads);
+}
+// `want` transforms of t threads each, or as many as make up a warp
+__host__ __device__ constexpr int per_block(int want, int t) { return want * t < 32 ? 32 / t : want; }
 
 // e^{-i pi j / N} for j = t + (N/R) q: in float tw[t] times the constant e^{-i pi q / R}
 // (one load per thread instead of R); in double (FP64-pipe bound) the table entry.
@@ -55,17 +72,18 @@ __host__ __device__ constexpr int row_sh() {
 // rows per block of the row passes and columns per block of the column pass
 template <typename T, int LOGN, int LOGR>
 __host__ __device__ constexpr int rows_per_block() {
-  constexpr int r = RegCfg<T, LOGR, 0>::MAXT / Plan<LOGN, LOGR>::T;
-  return r < 1 ? 1 : (r > (1 << LOGN) ? (1 << LOGN) : r);
+  constexpr int r = per_block(sizeof(T) == 4 || LOGN >= 9 ? 2 : 1, Plan<LOGN, LOGR>::T);
+  return r > (1 << LOGN) ? (1 << LOGN) : r;
 }
 template <typename T, int LOGM, int LOGR>
-__host__ __device__ constexpr int cols_per_block() {
-  constexpr int c = RegCfg<T, LOGR, 1>::MAXT / Plan<LOGM, LOGR>::T;
-  return c < 1 ? 1 : c;
-}
+__host__ __device__ constexpr int cols_per_block() { return per_block(1, Plan<LOGM, LOGR>::T); }
+template <typename T, int LOGN, int LOGR>
+__host__ __device__ constexpr int row_threads() { return rows_per_block<T, LOGN, LOGR>() * Plan<LOGN, LOGR>::T; }
+template <typename T, int LOGM, int LOGR>
+__host__ __device__ constexpr int col_threads() { return cols_per_block<T, LOGM, LOGR>() * Plan<LOGM, LOGR>::T; }
 
 template <typename T, int LOGN, int LOGR>
-__global__ void __launch_bounds__(RegCfg<T, LOGR, 0>::MAXT, RegCfg<T, LOGR, 0>::MINB)
+__global__ void __launch_bounds__((row_threads<T, LOGN, LOGR>()), (min_blocks(row_threads<T, LOGN, LOGR>(), RegCfg<T, LOGR, 0>::RES)))
 k_row_fwd_r(const T* __restrict__ p, cplx<T>* __restrict__ spec, const cplx<T>* __restrict__ twr,
             const cplx<T>* __restrict__ tw, const int* __restrict__ skip) {
   using C = cplx<T>;
@@ -143,7 +161,7 @@ k_row_fwd_r(const T* __restrict__ p, cplx<T>* __restrict__ spec, const cplx<T>* 
 }
 
 template <typename T, int LOGN, int LOGR>
-__global__ void __launch_bounds__(RegCfg<T, LOGR, 0>::MAXT, RegCfg<T, LOGR, 0>::MINB)
+__global__ void __launch_bounds__((row_threads<T, LOGN, LOGR>()), (min_blocks(row_threads<T, LOGN, LOGR>(), RegCfg<T, LOGR, 0>::RES)))
 k_row_inv_r(const cplx<T>* __restrict__ spec, T* __restrict__ u, const cplx<T>* __restrict__ twr,
             const cplx<T>* __restrict__ tw, const int* __restrict__ skip) {
   using C = cplx<T>;
@@ -219,7 +237,7 @@ k_row_inv_r(const cplx<T>* __restrict__ spec, T* __restrict__ u, const cplx<T>* 
 }
 
 template <typename T, int LOGM, int LOGR>
-__global__ void __launch_bounds__(RegCfg<T, LOGR, 1>::MAXT, RegCfg<T, LOGR, 1>::MINB)
+__global__ void __launch_bounds__((col_threads<T, LOGM, LOGR>()), (min_blocks(col_threads<T, LOGM, LOGR>(), RegCfg<T, LOGR, 1>::RES)))
 k_col_r(cplx<T>* __restrict__ spec, const T* __restrict__ table, const cplx<T>* __restrict__ twc, int nslots,
         const int* __restrict__ skip) {
   using C = cplx<T>;
@@ -261,17 +279,13 @@ k_col_r(cplx<T>* __restrict__ spec, const T* __restrict__ table, const cplx<T>* 
 // the length-2N FFT of the N nonzero rows (first stage pruned), times the pair of
 // compliances (tab2[pr (N + 1) + f] = (K(f, 2 pr), K(f, 2 pr + 1)) / M^2, f the folded
 // row wave number), the inverse FFT, the first N rows kept.
-template <int LOGR> struct ColPairCfg { static constexpr int MAXT = 256, MINB = 2; };
-template <> struct ColPairCfg<3> { static constexpr int MAXT = 512, MINB = 1; };
+template <int LOGM, int LOGR>
+__host__ __device__ constexpr int pairs_per_block() { return per_block(1, Plan<LOGM, LOGR>::T); }
+template <int LOGM, int LOGR>
+__host__ __device__ constexpr int pair_threads() { return pairs_per_block<LOGM, LOGR>() * Plan<LOGM, LOGR>::T; }
 
 template <int LOGM, int LOGR>
-__host__ __device__ constexpr int pairs_per_block() {
-  constexpr int c = ColPairCfg<LOGR>::MAXT / Plan<LOGM, LOGR>::T;
-  return c < 1 ? 1 : c;
-}
-
-template <int LOGM, int LOGR>
-__global__ void __launch_bounds__(ColPairCfg<LOGR>::MAXT, ColPairCfg<LOGR>::MINB)
+__global__ void __launch_bounds__((pair_threads<LOGM, LOGR>()), (min_blocks(pair_threads<LOGM, LOGR>(), kColPairRes)))
 k_col_p(float4* __restrict__ spec4, const float2* __restrict__ tab2, const float4* __restrict__ twp, int npairs,
         const int* __restrict__ skip) {
   using P = Plan<LOGM, LOGR>;

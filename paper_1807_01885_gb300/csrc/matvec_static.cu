@@ -142,6 +142,7 @@ extern "C" bem_status bem_matvec_static(const bem_kernel_desc* desc, const float
   while ((1 << k.logN) < N) ++k.logN;
   k.prec = BEM_FP32;
   k.elem = sizeof(float);
+  default_radix(&k);
   k.dev = dev;
   unsigned char* b = (unsigned char*)base;
   k.ws.spec = b + lay.spec;
