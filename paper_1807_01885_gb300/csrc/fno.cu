@@ -186,47 +186,6 @@ __global__ void k_pw(const float* __restrict__ X, const bf16* __restrict__ Wt, c
   }
 }
 
-// weight gradient partials: per block of FT pixels (of one sample) the Cout x Cin
-// products and the Cout bias sums; summed over blocks by k_pw_wgrad_sum
-__global__ void k_pw_wgrad(const float* __restrict__ dY, const float* __restrict__ X, float* __restrict__ part,
-                           int cout, int cin, size_t P) {
-  extern __shared__ float sh[];
-  float* dys = sh;                 // [cout][FT]
-  float* xs = sh + cout * FT;      // [cin][FT]
-  const int b = blockIdx.y;
-  const size_t p0 = blockIdx.x * (size_t)FT;
-  const int np = (int)std::min<size_t>(FT, P - p0);
-  for (int o = 0; o < cout; ++o)
-    dys[o * FT + threadIdx.x] = (int)threadIdx.x < np ? dY[((size_t)b * cout + o) * P + p0 + threadIdx.x] : 0.f;
-  for (int c = 0; c < cin; ++c)
-    xs[c * FT + threadIdx.x] = (int)threadIdx.x < np ? X[((size_t)b * cin + c) * P + p0 + threadIdx.x] : 0.f;
-  __syncthreads();
-  const size_t blk = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-  const int nout = cout * cin + cout;
-  for (int e = threadIdx.x; e < nout; e += blockDim.x) {
-    float acc = 0.f;
-    if (e < cout * cin) {
-      const int o = e / cin, c = e % cin;
-      for (int k = 0; k < FT; ++k) acc = fmaf(dys[o * FT + k], xs[c * FT + k], acc);
-    } else {
-      const int o = e - cout * cin;
-      for (int k = 0; k < FT; ++k) acc += dys[o * FT + k];
-    }
-    part[blk * nout + e] = acc;
-  }
-}
-
-__global__ void k_pw_wgrad_sum(const float* __restrict__ part, int nblk, int cout, int cin, float* __restrict__ gw,
-                               float* __restrict__ gb) {
-  const int nout = cout * cin + cout;
-  FOR_N(e, (size_t)nout) {
-    float acc = 0.f;
-    for (int k = 0; k < nblk; ++k) acc += part[(size_t)k * nout + e];
-    if (e < (size_t)cout * cin) gw[e] = acc;
-    else gb[e - (size_t)cout * cin] = acc;
-  }
-}
-
 __global__ void k_gelu_bwd(const float* __restrict__ dv, const float* __restrict__ z, float* __restrict__ dz, size_t n) {
   FOR_N(i, n) dz[i] = dv[i] * gelu_grad_f(z[i]);
 }
@@ -555,6 +514,8 @@ __global__ void __launch_bounds__(128) k_pw_tc(const float* __restrict__ X, int 
     }
   }
 }
+
+#include "fno_grad.cuh"
 
 // ---- fused Fourier layer (forward) --------------------------------------------
 // One kernel for z = W v + b + S(v) and v' = gelu(z): for 16 pixels y of one row x of
@@ -1376,9 +1337,8 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
     e = alloc(f, &f->TiB, (size_t)((2 * m + 15) / 16) * ((N + 7) / 8) * 32);
   if (e == cudaSuccess && fused_ok(f))
     e = alloc(f, &f->TfA, (size_t)((N + 15) / 16) * ((2 * m + 15) / 16) * 64);
-  const size_t nblk = (size_t)B * ((P + FT - 1) / FT);
   const size_t maxout = (size_t)std::max(W, H) * std::max({W, H, 7}) + std::max(W, H);
-  if (e == cudaSuccess && train) e = alloc(f, &f->part, nblk * maxout);
+  if (e == cudaSuccess && train) e = alloc(f, &f->part, kWgBlocks * maxout);
   if (e == cudaSuccess) e = alloc(f, &f->lpart, (size_t)4096);
   if (e == cudaSuccess) e = alloc(f, &f->cky, (size_t)m);
   if (e == cudaSuccess) e = alloc(f, &f->cky_s, (size_t)m);
@@ -1446,13 +1406,16 @@ bool width_ok(int c) { return c == 1 || c == 7 || c == 8 || c == 16 || c == 32 |
 
 void wgrad(const float* dY, int cout, const float* X, int cin, float* gw, float* gb, float* part, size_t P, int B,
            cudaStream_t s) {
-  static std::atomic<unsigned long long> attr{0};
-  if (first_on_device(attr)) cudaFuncSetAttribute(k_pw_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  dim3 grid((unsigned)((P + FT - 1) / FT), B);
-  const size_t sm = (size_t)(cout + cin) * FT * sizeof(float);
-  k_pw_wgrad<<<grid, FT, sm, s>>>(dY, X, part, cout, cin, P);
-  const int nblk = (int)(grid.x * grid.y);
-  k_pw_wgrad_sum<<<blocks_for((size_t)cout * cin + cout), FT, 0, s>>>(part, nblk, cout, cin, gw, gb);
+  const unsigned gps = (unsigned)((P + 31) / 32), groups = gps * (unsigned)B;
+  const int nblk = (int)std::min<unsigned>(kWgBlocks, (groups + 3) / 4);
+  const dim3 grid(nblk, 1, (unsigned)(((cout + 31) / 32) * ((cin + 31) / 32)));
+  // 16-byte loads where every row of both arrays starts on a 16-byte boundary (the
+  // features come from the caller and may lie anywhere)
+  const bool vec = P % 4 == 0 && ((uintptr_t)dY | (uintptr_t)X) % 16 == 0;
+  if (vec) k_pw_wgrad_tc<true><<<grid, 128, 0, s>>>(dY, X, part, cout, cin, (unsigned)P, gps, groups);
+  else k_pw_wgrad_tc<false><<<grid, 128, 0, s>>>(dY, X, part, cout, cin, (unsigned)P, gps, groups);
+  const int nw = cout * cin, nout = nw + cout;
+  k_pw_wgrad_sum<<<(nout + 31) / 32, 256, 0, s>>>(part, nblk, nw, nout, gw, gb);
   note_launches(2);
 }
 
