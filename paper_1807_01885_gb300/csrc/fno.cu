@@ -197,9 +197,9 @@ __device__ __forceinline__ int kx_of(int kxi, int m, int N) { return kxi < m ? k
 
 
 
-// A[bc][x][ky] = sum_kxi Y[bc][kxi][ky] e^{+2 pi i kx x/N}: one thread per (bc, x) and
-// four consecutive ky (one twiddle load serves four outputs)
-__global__ void k_idft_x(const float2* __restrict__ Y, float2* __restrict__ A, const float2* __restrict__ tw, int N,
+// A[bc][x][ky] = sum_kxi Y[bc][kxi][ky] e^{+2 pi i kx x/N} for any number of modes: one
+// thread per (bc, x) and four consecutive ky (one twiddle load serves four outputs)
+__global__ void k_idft_x_any(const float2* __restrict__ Y, float2* __restrict__ A, const float2* __restrict__ tw, int N,
                          int m, size_t bc) {
   const int mq = (m + 3) / 4;
   FOR_N(i, bc * (size_t)N * mq) {
@@ -1052,9 +1052,10 @@ __global__ void __launch_bounds__(256) k_idft_y_gemm(const float* __restrict__ A
   }
 }
 
-// Xh[q][kxi][ky] = s[ky] sum_x A[q][x][ky] e^{-2 pi i kx x/N}: block (q, kxi); thread
-// (slice, ky) adds every S-th x from its slice, then the slices are added in order
-__global__ void __launch_bounds__(256) k_dft_x_par(const float2* __restrict__ A, float2* __restrict__ Xh,
+// Xh[q][kxi][ky] = s[ky] sum_x A[q][x][ky] e^{-2 pi i kx x/N} for any number of modes:
+// block (q, kxi); thread (slice, ky) adds every S-th x from its slice, then the slices
+// are added in order
+__global__ void __launch_bounds__(256) k_dft_x_any(const float2* __restrict__ A, float2* __restrict__ Xh,
                                                    const float2* __restrict__ tw, const float* __restrict__ wky,
                                                    int N, int m) {
   __shared__ float2 red[256];
@@ -1092,24 +1093,7 @@ __global__ void __launch_bounds__(256) k_dft_x_par(const float2* __restrict__ A,
   }
 }
 
-// Y[b][o][mode] = sum_i X[b][i][mode] R[i][o][mode]
-__global__ void k_mix(const float2* __restrict__ X, const bf16* __restrict__ Rre, const bf16* __restrict__ Rim,
-                      float2* __restrict__ Y, int W, int nm, int B) {
-  FOR_N(e, (size_t)B * W * nm) {
-    const int mode = (int)(e % nm);
-    const int o = (int)((e / nm) % W);
-    const int b = (int)(e / ((size_t)nm * W));
-    float re = 0.f, im = 0.f;
-    for (int i = 0; i < W; ++i) {
-      const float2 x = X[((size_t)b * W + i) * nm + mode];
-      const size_t r = ((size_t)i * W + o) * nm + mode;
-      const float rr = b2f(Rre[r]), ri = b2f(Rim[r]);
-      re += x.x * rr - x.y * ri;
-      im += x.x * ri + x.y * rr;
-    }
-    Y[e] = make_float2(re, im);
-  }
-}
+#include "fno_modes.cuh"
 
 // dR[i][o][mode] = sum_b conj(X[b][i][mode]) dY[b][o][mode]
 __global__ void k_mix_wgrad(const float2* __restrict__ X, const float2* __restrict__ dY, float* __restrict__ gre,
@@ -1127,25 +1111,6 @@ __global__ void k_mix_wgrad(const float2* __restrict__ X, const float2* __restri
     }
     gre[e] = re;
     gim[e] = im;
-  }
-}
-
-// dX[b][i][mode] = sum_o conj(R[i][o][mode]) dY[b][o][mode]
-__global__ void k_mix_dgrad(const float2* __restrict__ dY, const bf16* __restrict__ Rre, const bf16* __restrict__ Rim,
-                            float2* __restrict__ dX, int W, int nm, int B) {
-  FOR_N(e, (size_t)B * W * nm) {
-    const int mode = (int)(e % nm);
-    const int i = (int)((e / nm) % W);
-    const int b = (int)(e / ((size_t)nm * W));
-    float re = 0.f, im = 0.f;
-    for (int o = 0; o < W; ++o) {
-      const float2 d = dY[((size_t)b * W + o) * nm + mode];
-      const size_t r = ((size_t)i * W + o) * nm + mode;
-      const float rr = b2f(Rre[r]), ri = b2f(Rim[r]);
-      re += rr * d.x + ri * d.y;
-      im += rr * d.y - ri * d.x;
-    }
-    dX[e] = make_float2(re, im);
   }
 }
 
@@ -1238,7 +1203,7 @@ struct bem_fno_s {
   float *a = nullptr, *h = nullptr, *out = nullptr, *dout = nullptr;
   float *dv = nullptr, *dz = nullptr, *dt = nullptr, *mom = nullptr, *part = nullptr, *cky = nullptr, *cky_s = nullptr;
   double* mom_part = nullptr;   // per-chunk sums of the height moments
-  float2 *A = nullptr, *Y = nullptr, *dY = nullptr, *tw = nullptr;
+  float2 *A = nullptr, *Y = nullptr, *dY = nullptr, *Xp = nullptr, *tw = nullptr, *twx = nullptr;
   float *Tf = nullptr, *Ti = nullptr;   // twiddle matrices of the y transforms (N x 2m, 2m x N)
   uint4 *TfB = nullptr, *TiB = nullptr; // the same split into bf16 hi/lo, in mma fragment order
   uint4* TfA = nullptr;                 // Tf split, in A-fragment order (fused layer kernel)
@@ -1284,7 +1249,8 @@ void set_twiddles(bem_fno_s* f, int N, cudaStream_t s) {
   k_twiddle_f<<<blocks_for(N), FT, 0, s>>>(f->tw, N);
   k_twiddle_mats<<<blocks_for((size_t)N * m), FT, 0, s>>>(f->tw, f->Tf, f->Ti, N, m);
   k_cky_scaled<<<1, 32, 0, s>>>(f->cky, f->cky_s, m, (float)(1.0 / ((double)N * N)));
-  note_launches(3);
+  k_twiddle_x<<<blocks_for((size_t)N * dft_x_kt(m)), FT, 0, s>>>(f->tw, f->twx, N, m);
+  note_launches(4);
   if (tc_ok(f)) {
     const int n2m = 2 * m;
     // forward B = Tf (K = N, columns n2m), inverse B = Ti (K = n2m, columns N)
@@ -1328,7 +1294,9 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
   if (e == cudaSuccess) e = alloc(f, &f->A, (size_t)B * W * N * m);
   if (e == cudaSuccess) e = alloc(f, &f->Y, (size_t)B * W * nm);
   if (e == cudaSuccess) e = alloc(f, &f->dY, (size_t)B * W * nm);
+  if (e == cudaSuccess) e = alloc(f, &f->Xp, (kXBlocks + (size_t)B * W) * nm);   // dft_x_chunks(bc) bc <= kXBlocks + bc
   if (e == cudaSuccess) e = alloc(f, &f->tw, (size_t)N);
+  if (e == cudaSuccess) e = alloc(f, &f->twx, (size_t)N * dft_x_kt(m));
   if (e == cudaSuccess) e = alloc(f, &f->Tf, (size_t)2 * m * N);
   if (e == cudaSuccess) e = alloc(f, &f->Ti, (size_t)2 * m * N);
   if (e == cudaSuccess && tc_ok(f))
@@ -1456,18 +1424,35 @@ void idft_y(bem_fno_s* f, float* out, const float* c, float scale, size_t rows, 
                                             n2m);
 }
 
+// X = truncated transform along x of A (scaled by wky), mixed over the channels by R
+// (CONJ: its adjoint) and back along x into A; X itself goes to Xh
+template <bool CONJ>
+void modes_x(bem_fno_s* f, int l, float2* Xh, const float* wky, int B, int N, cudaStream_t s) {
+  const int W = f->d.width, m = f->d.modes;
+  const size_t bc = (size_t)B * W, nm = 2 * (size_t)m * m;
+  const bf16* Rre = f->wb + f->o_Rre + (size_t)l * W * W * nm;
+  const bf16* Rim = f->wb + f->o_Rim + (size_t)l * W * W * nm;
+  const bool tiled = m <= kXModes;
+  const int chunks = tiled ? dft_x_chunks(bc, N) : 1;
+  float2* Xp = chunks > 1 ? f->Xp : Xh;
+  if (tiled) k_dft_x<<<dim3((unsigned)bc, chunks), 256, 0, s>>>(f->A, Xp, f->twx, wky, N, m);
+  else k_dft_x_any<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, Xp, f->tw, wky, N, m);
+  mix<CONJ>(Xp, chunks, Xh, Rre, Rim, f->Y, W, (int)nm, B, s);
+  if (tiled)
+    k_idft_x<<<dim3((unsigned)bc, (N + kXRows - 1) / kXRows), ((m + 1) / 2) * (kXRows / 4) > 128 ? 256 : 128,
+             idft_x_smem(m), s>>>(
+        f->Y, f->A, f->twx, N, m);
+  else
+    k_idft_x_any<<<blocks_for(bc * N * ((m + 3) / 4)), FT, 0, s>>>(f->Y, f->A, f->tw, N, m, bc);
+  note_launches(3);
+}
+
 // spectral branch up to the inverse along x: A[(b, o, x)][2m] holds the mixed modes
 // of every row, caching dft(vin) in Xh
 void spectral_modes(bem_fno_s* f, int l, const float* vin, float2* Xh, int B, int N, cudaStream_t s) {
-  const int W = f->d.width, m = f->d.modes;
-  const size_t bc = (size_t)B * W, nm = 2 * (size_t)m * m;
-  dft_y(f, vin, bc * N, N, s);
-  k_dft_x_par<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, Xh, f->tw, nullptr, N, m);
-  const bf16* Rre = f->wb + f->o_Rre + (size_t)l * W * W * nm;
-  const bf16* Rim = f->wb + f->o_Rim + (size_t)l * W * W * nm;
-  k_mix<<<blocks_for(bc * nm), FT, 0, s>>>(Xh, Rre, Rim, f->Y, W, (int)nm, B);
-  k_idft_x<<<blocks_for(bc * N * ((m + 3) / 4)), FT, 0, s>>>(f->Y, f->A, f->tw, N, m, bc);
-  note_launches(4);
+  dft_y(f, vin, (size_t)B * f->d.width * N, N, s);
+  note_launches(1);
+  modes_x<false>(f, l, Xh, nullptr, B, N, s);
 }
 
 void spectral_fwd(bem_fno_s* f, int l, const float* vin, float2* Xh, float* out, int B, int N, cudaStream_t s) {
@@ -1605,16 +1590,12 @@ bem_status backward(bem_fno_s* f, int B, int N, const float* x, const float* tar
     pw<true, false, false>(dz, W, f->wb + f->o_Ww + (size_t)l * W * W, nullptr, f->dt, nullptr, W, P, B, s);
     // spectral branch: dY = (c/N^2) dft(dz); dR = sum_b conj(Xh) dY; dXh = sum_o conj(R) dY
     dft_y(f, dz, bc * N, N, s);
-    k_dft_x_par<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, f->dY, f->tw, f->cky_s, N, m);
-    const bf16* Rre = f->wb + f->o_Rre + (size_t)l * W * W * nm;
-    const bf16* Rim = f->wb + f->o_Rim + (size_t)l * W * W * nm;
+    // (and d_vin += Re(sum dXh e^{+i theta}), the adjoint of the forward transform)
+    modes_x<true>(f, l, f->dY, f->cky_s, B, N, s);
     k_mix_wgrad<<<blocks_for((size_t)W * W * nm), FT, 0, s>>>(f->Xh[l], f->dY, f->g + f->o_Rre + (size_t)l * W * W * nm,
                                                           f->g + f->o_Rim + (size_t)l * W * W * nm, W, (int)nm, B);
-    k_mix_dgrad<<<blocks_for(bc * nm), FT, 0, s>>>(f->dY, Rre, Rim, f->Y, W, (int)nm, B);
-    // d_vin += Re(sum dXh e^{+i theta}) (adjoint of the forward transform)
-    k_idft_x<<<blocks_for(bc * N * ((m + 3) / 4)), FT, 0, s>>>(f->Y, f->A, f->tw, N, m, bc);
     idft_y<true>(f, f->dt, nullptr, 1.f, bc * N, N, s);
-    note_launches(6);
+    note_launches(3);
     std::swap(f->dv, f->dt);
   }
   wgrad(f->dv, W, x, 7, f->g + f->o_Pw, f->g + f->o_Pb, f->part, P, B, s);

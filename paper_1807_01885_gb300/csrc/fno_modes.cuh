@@ -7,14 +7,28 @@
 // the arithmetic is small and the work is in feeding it.  Wave numbers come in pairs
 // +-k that share their products with cos and sin, which halves the multiply-adds, and
 // each thread keeps a register tile (2 ky x 4 k, or 2 ky x 4 x), so that one 16-byte and
-// four 8-byte shared-memory reads serve 32 multiply-adds.  (One thread per output and a
-// twiddle load from global memory per product took 80 and 60 us for 512 channels of
-// N = 256, m = 16, where reading and writing the arrays takes 5 us.)
+// four 8-byte shared-memory reads serve 32 multiply-adds.
+// The twiddles come from a table in the order of use, twx[x][k] = tw[k x mod N] for k in
+// [0, m] (rows of dft_x_kt(m), the rest 0), so that staging them is a plain copy.
+// (One thread per output and a twiddle load per product took 80 and 60 us for 512 channels
+// of N = 256, m = 16; twiddles gathered by every block 28 and 20 us.)
 #pragma once
 
 constexpr int kXRows = 64;        // rows x staged in shared memory at a time
 constexpr int kXModes = 32;       // most modes per axis that the tiled kernels take
-constexpr int kXBlocks = 456;     // blocks that fill the GPU (three per SM)
+constexpr int kXBlocks = 912;     // blocks that fill the GPU (six per SM)
+
+// row length of the twiddle table: k in [0, m], rounded up to groups of four
+__host__ __device__ inline int dft_x_kt(int m) { return 4 * ((m + 4) / 4); }
+
+__global__ void k_twiddle_x(const float2* __restrict__ tw, float2* __restrict__ twx, int N, int m) {
+  const int kt = dft_x_kt(m);
+  FOR_N(i, (size_t)N * kt) {
+    const unsigned k = (unsigned)(i % kt);
+    const size_t x = i / kt;
+    twx[i] = (int)k <= m ? tw[(k * x) % (size_t)N] : make_float2(0.f, 0.f);
+  }
+}
 
 // blocks per channel along x of k_dft_x (each adds its share of the rows)
 inline int dft_x_chunks(size_t bc, int N) {
@@ -24,10 +38,10 @@ inline int dft_x_chunks(size_t bc, int N) {
 
 // Xp[chunk][q][kxi][ky] = wky[ky] sum over the chunk's rows x of A[q][x][ky] e^{-2 pi i kx x / N}
 __global__ void __launch_bounds__(256) k_dft_x(const float2* __restrict__ A, float2* __restrict__ Xp,
-                                               const float2* __restrict__ tw, const float* __restrict__ wky, int N,
+                                               const float2* __restrict__ twx, const float* __restrict__ wky, int N,
                                                int m) {
   __shared__ __align__(16) float smem[kXRows * (kXModes * 2 + 36 * 2)];
-  const int ky2 = (m + 1) / 2, kg = (m + 4) / 4, kt = 4 * kg, items = ky2 * kg, S = 256 / items;
+  const int ky2 = (m + 1) / 2, kg = (m + 4) / 4, kt = dft_x_kt(m), items = ky2 * kg, S = 256 / items;
   float2* const sA = reinterpret_cast<float2*>(smem);                  // [kXRows][2 ky2]
   float2* const sT = sA + kXRows * 2 * ky2;                            // [kXRows][kt]
   const size_t q = blockIdx.x;
@@ -40,14 +54,17 @@ __global__ void __launch_bounds__(256) k_dft_x(const float2* __restrict__ A, flo
   for (int tile = t0; tile < t1; ++tile) {
     const int x0 = tile * kXRows, nx = min(kXRows, N - x0);
     __syncthreads();
-    for (int e = tid; e < nx * 2 * ky2; e += 256) {
-      const int x = e / (2 * ky2), ky = e - x * 2 * ky2;
-      sA[e] = ky < m ? A[(q * N + x0 + x) * m + ky] : make_float2(0.f, 0.f);
+    if (m % 2 == 0) {
+      const float4* a = reinterpret_cast<const float4*>(A + (q * N + x0) * m);
+      for (int e = tid; e < nx * ky2; e += 256) reinterpret_cast<float4*>(sA)[e] = a[e];
+    } else {
+      for (int e = tid; e < nx * 2 * ky2; e += 256) {
+        const int x = e / (2 * ky2), ky = e - x * 2 * ky2;
+        sA[e] = ky < m ? A[(q * N + x0 + x) * m + ky] : make_float2(0.f, 0.f);
+      }
     }
-    for (int e = tid; e < nx * kt; e += 256) {
-      const int x = e / kt, k = e - x * kt;
-      sT[e] = k <= m ? tw[((unsigned)k * (unsigned)(x0 + x)) % (unsigned)N] : make_float2(0.f, 0.f);
-    }
+    for (int e = tid; e < nx * kt / 2; e += 256)
+      reinterpret_cast<float4*>(sT)[e] = reinterpret_cast<const float4*>(twx + (size_t)x0 * kt)[e];
     __syncthreads();
     if (slice < S) {
       for (int x = slice; x < nx; x += S) {
@@ -97,13 +114,16 @@ __global__ void __launch_bounds__(256) k_dft_x(const float2* __restrict__ A, flo
 }
 
 // A[q][x][ky] = sum_kxi Y[q][kxi][ky] e^{+2 pi i kx x / N}: block (channel, kXRows rows)
+inline size_t idft_x_smem(int m) {
+  return (size_t)(m + 1) * (2 * ((m + 1) / 2)) * sizeof(float4) + (size_t)kXRows * dft_x_kt(m) * sizeof(float2);
+}
 __global__ void __launch_bounds__(256) k_idft_x(const float2* __restrict__ Y, float2* __restrict__ A,
-                                                const float2* __restrict__ tw, int N, int m) {
-  __shared__ __align__(16) float4 sY[(kXModes + 1) * kXModes];   // per k and ky: Y+ + Y-, Y+ - Y-
-  __shared__ float2 sT[(kXModes + 1) * kXRows];                   // [k][x]
+                                                const float2* __restrict__ twx, int N, int m) {
+  extern __shared__ __align__(16) float4 sY[];                    // [m + 1][2 ky2]: Y+ + Y-, Y+ - Y-
   const size_t q = blockIdx.x;
   const int x0 = blockIdx.y * kXRows, nx = min(kXRows, N - x0);
-  const int ky2 = (m + 1) / 2, row = 2 * ky2;
+  const int ky2 = (m + 1) / 2, row = 2 * ky2, kt = dft_x_kt(m);
+  float2* const sT = reinterpret_cast<float2*>(sY + (m + 1) * row);   // [x][kt]
   const float2* y = Y + q * 2 * m * m;
   for (int e = threadIdx.x; e < (m + 1) * row; e += blockDim.x) {
     const int k = e / row, ky = e - k * row;
@@ -111,10 +131,8 @@ __global__ void __launch_bounds__(256) k_idft_x(const float2* __restrict__ Y, fl
     const float2 b = (k > 0 && ky < m) ? y[(2 * m - k) * m + ky] : make_float2(0.f, 0.f);
     sY[e] = make_float4(a.x + b.x, a.y + b.y, a.x - b.x, a.y - b.y);
   }
-  for (int e = threadIdx.x; e < (m + 1) * kXRows; e += blockDim.x) {
-    const int k = e / kXRows, x = min(e - k * kXRows, nx - 1);
-    sT[e] = tw[((unsigned)k * (unsigned)(x0 + x)) % (unsigned)N];
-  }
+  for (int e = threadIdx.x; e < nx * kt / 2; e += blockDim.x)
+    reinterpret_cast<float4*>(sT)[e] = reinterpret_cast<const float4*>(twx + (size_t)x0 * kt)[e];
   __syncthreads();
   for (int it = threadIdx.x; it < ky2 * (kXRows / 4); it += blockDim.x) {
     const int kyp = it % ky2, xl = 4 * (it / ky2);
@@ -122,9 +140,13 @@ __global__ void __launch_bounds__(256) k_idft_x(const float2* __restrict__ Y, fl
     float o[4][4] = {};
     for (int k = 0; k <= m; ++k) {
       const float4 y0 = sY[k * row + 2 * kyp], y1 = sY[k * row + 2 * kyp + 1];
-      const float4* tp = reinterpret_cast<const float4*>(sT + k * kXRows + xl);
-      const float4 wa = tp[0], wb = tp[1];
-      const float wx[4] = {wa.x, wa.z, wb.x, wb.z}, wy[4] = {wa.y, wa.w, wb.y, wb.w};
+      float wx[4], wy[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 w = sT[min(xl + e, nx - 1) * kt + k];
+        wx[e] = w.x;
+        wy[e] = w.y;
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         o[e][0] = fmaf(y0.w, wy[e], fmaf(y0.x, wx[e], o[e][0]));
@@ -206,9 +228,8 @@ __global__ void __launch_bounds__(256) k_mix(const float2* __restrict__ Xp, int 
 template <bool CONJ>
 void mix(const float2* Xp, int chunks, float2* Xh, const bf16* Rre, const bf16* Rim, float2* Y, int W, int nm, int B,
          cudaStream_t s) {
-  // four outputs per warp read each mode of X once for all; one where that leaves the
-  // GPU with few blocks (a single sample of 512 modes: 16 blocks against 64)
+  // two outputs per warp; one where that leaves the GPU with few blocks
   const dim3 g((nm + 31) / 32, (B + kMixB - 1) / kMixB);
-  if (g.x * g.y >= 64) k_mix<4, CONJ><<<dim3(g.x, g.y, (W + 31) / 32), 256, 0, s>>>(Xp, chunks, Xh, Rre, Rim, Y, W, nm, B);
+  if (g.x * g.y >= 128) k_mix<2, CONJ><<<dim3(g.x, g.y, (W + 15) / 16), 256, 0, s>>>(Xp, chunks, Xh, Rre, Rim, Y, W, nm, B);
   else k_mix<1, CONJ><<<dim3(g.x, g.y, (W + 7) / 8), 256, 0, s>>>(Xp, chunks, Xh, Rre, Rim, Y, W, nm, B);
 }
