@@ -72,6 +72,35 @@ __device__ __forceinline__ void gelu2(float& z0, float& z1) {
   gup(u, u0, u1);
   gup(gmul(gmul(z, gsplat(0.5f)), gpk(u0 >= 0.f ? 2.f - y0 : y0, u1 >= 0.f ? 2.f - y1 : y1)), z0, z1);
 }
+// gelu'(z) = Phi(z) + z phi(z) of two values and gelu(z) = z Phi(z) beside it, by erfc(u) =
+// t P(t) e^{-u^2}, t = 1 / (1 + 0.4 u): the same form with one term more, coefficients by a
+// minimax fit (linear programming on u in [0, 6], error below 1e-8; in float arithmetic
+// 4e-8 rms): the 1.5e-7 of the shorter one is a bias that adds up over the pixels of a
+// gradient.  e^{-u^2} is also the density's e^{-z^2/2}.
+__device__ __forceinline__ void gelu_both2(float z0, float z1, float& h0, float& h1, float& d0, float& d1) {
+  const g2x z = gpk(z0, z1);
+  const g2x u = gmul(z, gsplat(0.70710678118654752f));
+  const g2x a = u & 0x7fffffff7fffffffull;
+  float r0, r1;
+  gup(gfma(a, gsplat(0.4f), gsplat(1.f)), r0, r1);
+  const g2x t = gpk(__fdividef(1.f, r0), __fdividef(1.f, r1));
+  g2x y = gfma(t, gsplat(-0.20324541657427708f), gsplat(0.7213278152423136f));
+  y = gfma(t, y, gsplat(-0.3906169638412854f));
+  y = gfma(t, y, gsplat(0.4840823859374485f));
+  y = gfma(t, y, gsplat(0.15554031289499895f));
+  y = gfma(t, y, gsplat(0.23291186634080138f));
+  float q0, q1;
+  gup(gmul(a, a), q0, q1);
+  const g2x ex = gpk(__expf(-q0), __expf(-q1));
+  y = gmul(gmul(t, y), ex);
+  float y0, y1, u0, u1;
+  gup(y, y0, y1);
+  gup(u, u0, u1);
+  const g2x phi2 = gpk(u0 >= 0.f ? 2.f - y0 : y0, u1 >= 0.f ? 2.f - y1 : y1);   // 2 Phi(z)
+  const g2x Phi = gmul(phi2, gsplat(0.5f));
+  gup(gmul(z, Phi), h0, h1);
+  gup(gfma(gmul(z, gsplat(0.39894228040143268f)), ex, Phi), d0, d1);
+}
 __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
@@ -548,11 +577,37 @@ __global__ void k_frag_a(const float* __restrict__ Am, int M, int K, size_t ldr,
   }
 }
 
+// The two contractions of the backward layer.  The unit's accumulators truncate, a bias
+// that adds up over the pixels of a gradient (the bias gradient of the lift: 1.2e-6 with
+// one ten-step accumulator against 0.5e-6): each contraction has its own, the small terms
+// come first and the two are added in float.
+template <int KT, int KS, int NT>
+__device__ __forceinline__ void layer_product_bwd(float (&acc)[4], const unsigned (&ah)[KT][4],
+                                                  const unsigned (&al)[KT][4], const unsigned (&th)[KS][4],
+                                                  const unsigned (&tl)[KS][4], const unsigned (&wf)[KT][NT][2],
+                                                  const unsigned (&sfh)[KS][NT][2],
+                                                  const unsigned (&sfl)[KS][NT][2], int nt) {
+  float m[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int kb = 0; kb < KT; ++kb) mma_bf16(acc, al[kb], wf[kb][nt][0], wf[kb][nt][1]);
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) {
+    mma_bf16(m, th[ks], sfl[ks][nt][0], sfl[ks][nt][1]);
+    mma_bf16(m, tl[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+  }
+#pragma unroll
+  for (int kb = 0; kb < KT; ++kb) mma_bf16(acc, ah[kb], wf[kb][nt][0], wf[kb][nt][1]);
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) mma_bf16(m, th[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) acc[e] += m[e];
+}
+
 // NT n-tiles of the outputs (width W = 8 NT), KT = ceil(W / 16) k-blocks of the channel
 // contraction, KS k-blocks of the modes (2m <= 16 KS).  Warp w of the grid takes row
 // (b, x) = w / chunks and the y-tiles [chunk * tpw, (chunk + 1) * tpw).  Offsets
 // within one sample are 32-bit (W N^2 < 2^31).
-template <int KT, int NT, int KS>
+template <int KT, int NT, int KS, bool BWD>
 __global__ void __launch_bounds__(128) k_layer_tc(const float* __restrict__ V, const bf16* __restrict__ Ww,
                                                   const bf16* __restrict__ bias, const float* __restrict__ A,
                                                   const float* __restrict__ cs, const uint4* __restrict__ TfA,
@@ -579,8 +634,8 @@ __global__ void __launch_bounds__(128) k_layer_tc(const float* __restrict__ V, c
       for (int hh = 0; hh < 2; ++hh) {
         const int c = 16 * kb + 2 * t + 8 * hh;
         const bool cv = 16 * kb + 8 * hh < W;   // c < W for every lane, or for none
-        const unsigned lo = cv ? (unsigned)__bfloat16_as_ushort(Ww[o * W + c]) : 0u;
-        const unsigned hi = cv ? (unsigned)__bfloat16_as_ushort(Ww[o * W + c + 1]) : 0u;
+        const unsigned lo = cv ? (unsigned)__bfloat16_as_ushort(Ww[BWD ? c * W + o : o * W + c]) : 0u;
+        const unsigned hi = cv ? (unsigned)__bfloat16_as_ushort(Ww[BWD ? (c + 1) * W + o : o * W + c + 1]) : 0u;
         wf[kb][nt][hh] = lo | (hi << 16);
       }
     }
@@ -594,8 +649,8 @@ __global__ void __launch_bounds__(128) k_layer_tc(const float* __restrict__ V, c
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
         const int k = 16 * ks + 2 * t + 8 * hh;
-        const float x0 = k < n2m ? ar[k] * cs[k / 2] : 0.f;
-        const float x1 = k + 1 < n2m ? ar[k + 1] * cs[(k + 1) / 2] : 0.f;
+        const float x0 = k < n2m ? (BWD ? ar[k] : ar[k] * cs[k / 2]) : 0.f;
+        const float x1 = k + 1 < n2m ? (BWD ? ar[k + 1] : ar[k + 1] * cs[(k + 1) / 2]) : 0.f;
         split2(x0, x1, sfh[ks][nt][hh], sfl[ks][nt][hh]);
       }
     }
@@ -641,28 +696,41 @@ __global__ void __launch_bounds__(128) k_layer_tc(const float* __restrict__ V, c
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      if constexpr (BWD) {
+        layer_product_bwd<KT, KS>(acc, ah, al, th, tl, wf, sfh, sfl, nt);
+      } else {
 #pragma unroll
-      for (int kb = 0; kb < KT; ++kb) {
-        mma_bf16(acc, ah[kb], wf[kb][nt][0], wf[kb][nt][1]);
-        mma_bf16(acc, al[kb], wf[kb][nt][0], wf[kb][nt][1]);
-      }
+        for (int kb = 0; kb < KT; ++kb) {
+          mma_bf16(acc, ah[kb], wf[kb][nt][0], wf[kb][nt][1]);
+          mma_bf16(acc, al[kb], wf[kb][nt][0], wf[kb][nt][1]);
+        }
 #pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        mma_bf16(acc, th[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
-        mma_bf16(acc, th[ks], sfl[ks][nt][0], sfl[ks][nt][1]);
-        mma_bf16(acc, tl[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+        for (int ks = 0; ks < KS; ++ks) {
+          mma_bf16(acc, th[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+          mma_bf16(acc, th[ks], sfl[ks][nt][0], sfl[ks][nt][1]);
+          mma_bf16(acc, tl[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+        }
       }
       // acc[0], acc[1]: pixel ya, outputs o0, o0 + 1; acc[2], acc[3]: pixel yb
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const unsigned oo = (unsigned)(8 * nt + 2 * t + e) * P;
         const float va = acc[e] + bv[nt][e], vb2 = acc[2 + e] + bv[nt][e];
-        if (zb != nullptr) {
-          if (oka) zb[oo + ya] = va;
-          if (okb) zb[oo + yb] = vb2;
-        }
         float wa = va, wb = vb2;
-        if (gelu) gelu2(wa, wb);
+        if constexpr (BWD) {
+          if (zb != nullptr) {
+            float h0, h1, d0, d1;
+            gelu_both2(oka ? zb[oo + ya] : 0.f, okb ? zb[oo + yb] : 0.f, h0, h1, d0, d1);
+            wa *= d0;
+            wb *= d1;
+          }
+        } else {
+          if (zb != nullptr) {
+            if (oka) zb[oo + ya] = va;
+            if (okb) zb[oo + yb] = vb2;
+          }
+          if (gelu) gelu2(wa, wb);
+        }
         if (oka) ub[oo + ya] = wa;
         if (okb) ub[oo + yb] = wb;
       }
@@ -689,9 +757,15 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // flight while one is contracted; four stages measured no faster, the kernel being
 // bound by its instruction issue): each warp stages its W channels x 16 pixels (W
 // 64-byte rows, row stride 20 floats, which makes the fragment reads conflict-free).
-// Same arithmetic and order as k_layer_tc.
+// Same arithmetic and order as k_layer_tc.  BWD (both kernels): the layer's data gradient
+// d v = W^T dz + adjoint of S: V is dz, the weights are read transposed, A holds the
+// x-inverse of the adjoint's modes (weight 1), and where Z is given (the previous
+// layer's pre-activations) the result is multiplied by gelu'(Z), which makes it that
+// layer's dz.  One pass over the pixels where the separate kernels (gelu', W^T dz, the
+// inverse y-transform added in place) took three more reads and two more writes of the
+// activations: 850 -> 440 us per gradient pass of 16 x 256 x 256, four layers (GB300).
 constexpr int kLayerRow = 20, kLayerStages = 2;
-template <int KT, int NT, int KS>
+template <int KT, int NT, int KS, bool BWD>
 __global__ void __launch_bounds__(128, 4) k_layer_tc_pipe(const float* __restrict__ V, const bf16* __restrict__ Ww,
                                                        const bf16* __restrict__ bias, const float* __restrict__ A,
                                                        const float* __restrict__ cs, const uint4* __restrict__ TfA,
@@ -718,8 +792,8 @@ __global__ void __launch_bounds__(128, 4) k_layer_tc_pipe(const float* __restric
       for (int hh = 0; hh < 2; ++hh) {
         const int c = 16 * kb + 2 * t + 8 * hh;
         const bool cv = 16 * kb + 8 * hh < W;
-        const unsigned lo = cv ? (unsigned)__bfloat16_as_ushort(Ww[o * W + c]) : 0u;
-        const unsigned hi = cv ? (unsigned)__bfloat16_as_ushort(Ww[o * W + c + 1]) : 0u;
+        const unsigned lo = cv ? (unsigned)__bfloat16_as_ushort(Ww[BWD ? c * W + o : o * W + c]) : 0u;
+        const unsigned hi = cv ? (unsigned)__bfloat16_as_ushort(Ww[BWD ? (c + 1) * W + o : o * W + c + 1]) : 0u;
         wf[kb][nt][hh] = lo | (hi << 16);
       }
     }
@@ -733,8 +807,8 @@ __global__ void __launch_bounds__(128, 4) k_layer_tc_pipe(const float* __restric
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
         const int k = 16 * ks + 2 * t + 8 * hh;
-        const float x0 = k < n2m ? ar[k] * cs[k / 2] : 0.f;
-        const float x1 = k + 1 < n2m ? ar[k + 1] * cs[(k + 1) / 2] : 0.f;
+        const float x0 = k < n2m ? (BWD ? ar[k] : ar[k] * cs[k / 2]) : 0.f;
+        const float x1 = k + 1 < n2m ? (BWD ? ar[k + 1] : ar[k + 1] * cs[(k + 1) / 2]) : 0.f;
         split2(x0, x1, sfh[ks][nt][hh], sfl[ks][nt][hh]);
       }
     }
@@ -791,6 +865,19 @@ __global__ void __launch_bounds__(128, 4) k_layer_tc_pipe(const float* __restric
       for (int r = 0; r < 4; ++r) split2(xv[r][0], xv[r][1], ah[kb][r], al[kb][r]);
     }
     __syncwarp();   // every lane has read the stage before it is refilled
+    [[maybe_unused]] float zv[BWD ? NT : 1][4];   // this tile's pre-activations, loaded ahead of the products
+    if constexpr (BWD) {
+      if (zb != nullptr) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const unsigned oo = (unsigned)(8 * nt + 2 * t + e) * P;
+            zv[nt][e] = zb[oo + ya];
+            zv[nt][2 + e] = zb[oo + yb];
+          }
+      }
+    }
     unsigned th[KS][4], tl[KS][4];
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
@@ -802,27 +889,40 @@ __global__ void __launch_bounds__(128, 4) k_layer_tc_pipe(const float* __restric
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      if constexpr (BWD) {
+        layer_product_bwd<KT, KS>(acc, ah, al, th, tl, wf, sfh, sfl, nt);
+      } else {
 #pragma unroll
-      for (int kb = 0; kb < KT; ++kb) {
-        mma_bf16(acc, ah[kb], wf[kb][nt][0], wf[kb][nt][1]);
-        mma_bf16(acc, al[kb], wf[kb][nt][0], wf[kb][nt][1]);
-      }
+        for (int kb = 0; kb < KT; ++kb) {
+          mma_bf16(acc, ah[kb], wf[kb][nt][0], wf[kb][nt][1]);
+          mma_bf16(acc, al[kb], wf[kb][nt][0], wf[kb][nt][1]);
+        }
 #pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        mma_bf16(acc, th[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
-        mma_bf16(acc, th[ks], sfl[ks][nt][0], sfl[ks][nt][1]);
-        mma_bf16(acc, tl[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+        for (int ks = 0; ks < KS; ++ks) {
+          mma_bf16(acc, th[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+          mma_bf16(acc, th[ks], sfl[ks][nt][0], sfl[ks][nt][1]);
+          mma_bf16(acc, tl[ks], sfh[ks][nt][0], sfh[ks][nt][1]);
+        }
       }
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const unsigned oo = (unsigned)(8 * nt + 2 * t + e) * P;
         const float va = acc[e] + bv[nt][e], vb2 = acc[2 + e] + bv[nt][e];
-        if (zb != nullptr) {
-          zb[oo + ya] = va;
-          zb[oo + yb] = vb2;
-        }
         float wa = va, wb = vb2;
-        if (gelu) gelu2(wa, wb);
+        if constexpr (BWD) {
+          if (zb != nullptr) {
+            float h0, h1, d0, d1;
+            gelu_both2(zv[nt][e], zv[nt][2 + e], h0, h1, d0, d1);
+            wa *= d0;
+            wb *= d1;
+          }
+        } else {
+          if (zb != nullptr) {
+            zb[oo + ya] = va;
+            zb[oo + yb] = vb2;
+          }
+          if (gelu) gelu2(wa, wb);
+        }
         ub[oo + ya] = wa;
         ub[oo + yb] = wb;
       }
@@ -1461,30 +1561,30 @@ void spectral_fwd(bem_fno_s* f, int l, const float* vin, float2* Xh, float* out,
   note_launches(1);
 }
 
-template <int KT, int NT, int KS>
+template <int KT, int NT, int KS, bool BWD>
 void layer_launch(bem_fno_s* f, const float* vin, const bf16* Ww, const bf16* Wb, float* z, float* vout, bool gelu,
                   int B, int N, cudaStream_t s) {
   const int YT = (N + 15) / 16, tpw = std::min(YT, 32), chunks = (YT + tpw - 1) / tpw;
   const size_t rows = (size_t)B * N, warps = rows * chunks;
   if (N % 16 == 0) {   // whole 16-pixel tiles, 16-byte aligned rows: the staged form
-    k_layer_tc_pipe<KT, NT, KS><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(
+    k_layer_tc_pipe<KT, NT, KS, BWD><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(
         vin, Ww, Wb, reinterpret_cast<const float*>(f->A), f->cky_s, f->TfA, z, vout, N, 2 * f->d.modes, rows, tpw,
         gelu ? 1 : 0);
     return;
   }
-  k_layer_tc<KT, NT, KS><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(
+  k_layer_tc<KT, NT, KS, BWD><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(
       vin, Ww, Wb, reinterpret_cast<const float*>(f->A), f->cky_s, f->TfA, z, vout, N, 2 * f->d.modes, rows, tpw,
       gelu ? 1 : 0);
 }
 
-template <int KT, int NT>
+template <int KT, int NT, bool BWD>
 void layer_ks(bem_fno_s* f, const float* vin, const bf16* Ww, const bf16* Wb, float* z, float* vout, bool gelu, int B,
               int N, cudaStream_t s) {
   switch ((2 * f->d.modes + 15) / 16) {
-    case 1: layer_launch<KT, NT, 1>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
-    case 2: layer_launch<KT, NT, 2>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
-    case 3: layer_launch<KT, NT, 3>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
-    default: layer_launch<KT, NT, 4>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
+    case 1: layer_launch<KT, NT, 1, BWD>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
+    case 2: layer_launch<KT, NT, 2, BWD>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
+    case 3: layer_launch<KT, NT, 3, BWD>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
+    default: layer_launch<KT, NT, 4, BWD>(f, vin, Ww, Wb, z, vout, gelu, B, N, s); break;
   }
 }
 
@@ -1496,10 +1596,25 @@ void layer_fused(bem_fno_s* f, int l, const float* vin, float2* Xh, float* z, fl
   spectral_modes(f, l, vin, Xh, B, N, s);
   const bf16* Ww = f->wb + f->o_Ww + (size_t)l * W * W;
   const bf16* Wb = f->wb + f->o_Wb + (size_t)l * W;
-  if (W == 8) layer_ks<1, 1>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
-  else if (W == 16) layer_ks<1, 2>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
-  else layer_ks<2, 4>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
+  if (W == 8) layer_ks<1, 1, false>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
+  else if (W == 16) layer_ks<1, 2, false>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
+  else layer_ks<2, 4, false>(f, vin, Ww, Wb, z, vout, gelu, B, N, s);
   note_launches(1);
+}
+
+// dv = W^T dz + adjoint of S (its modes along x already in A), times gelu'(zprev) where
+// it is given (fused_ok)
+void layer_fused_bwd(bem_fno_s* f, int l, const float* dz, float* zprev, float* dv, int B, int N, cudaStream_t s) {
+  const int W = f->d.width;
+  const bf16* Ww = f->wb + f->o_Ww + (size_t)l * W * W;
+  if (W == 8) layer_ks<1, 1, true>(f, dz, Ww, nullptr, zprev, dv, false, B, N, s);
+  else if (W == 16) layer_ks<1, 2, true>(f, dz, Ww, nullptr, zprev, dv, false, B, N, s);
+  else layer_ks<2, 4, true>(f, dz, Ww, nullptr, zprev, dv, false, B, N, s);
+  note_launches(1);
+}
+
+bool fused_size(const bem_fno_s* f, int N) {   // 32-bit offsets within a sample
+  return fused_ok(f) && (size_t)f->d.width * N * N < (size_t(1) << 32);
 }
 
 template <int KT, int NT>
@@ -1537,9 +1652,9 @@ bem_status forward(bem_fno_s* f, int B, int N, const float* x, bool train, cudaS
     float* z = train ? f->z[l] : f->z[0];
     float2* Xh = train ? f->Xh[l] : f->Xh[0];
     float* vout = train ? f->v[l + 1] : f->v[(l + 1) & 1];
-    if (fused_ok(f) && (size_t)W * P < (size_t(1) << 32)) {   // 32-bit offsets within a sample
-      // z is kept only for the backward pass
-      layer_fused(f, l, vin, Xh, train ? z : nullptr, vout, l < L - 1, B, N, s);
+    if (fused_size(f, N)) {
+      // z is kept only for the backward pass, which needs it where a gelu follows
+      layer_fused(f, l, vin, Xh, train && l < L - 1 ? z : nullptr, vout, l < L - 1, B, N, s);
       continue;
     }
     spectral_fwd(f, l, vin, Xh, z, B, N, s);
@@ -1569,8 +1684,6 @@ bem_status backward(bem_fno_s* f, int B, int N, const float* x, const float* tar
   const int lb = std::min(blocks_for((size_t)B * P), 4096);
   k_mse<<<lb, FT, 0, s>>>(f->out, target, f->dout, f->lpart, (size_t)B * P);
   note_launches(1);
-  std::vector<double> lp(lb);
-  BEM_CUDA_TRY(cudaMemcpyAsync(lp.data(), f->lpart, lb * sizeof(double), cudaMemcpyDeviceToHost, s));
   // projection
   wgrad(f->dout, 1, f->h, H, f->g + f->o_Q2w, f->g + f->o_Q2b, f->part, P, B, s);
   pw<true, false, false>(f->dout, 1, f->wb + f->o_Q2w, nullptr, f->dt, nullptr, H, P, B, s);   // d_h
@@ -1579,27 +1692,38 @@ bem_status backward(bem_fno_s* f, int B, int N, const float* x, const float* tar
   wgrad(f->dz, H, f->v[L], W, f->g + f->o_Q1w, f->g + f->o_Q1b, f->part, P, B, s);
   pw<true, false, false>(f->dz, H, f->wb + f->o_Q1w, nullptr, f->dv, nullptr, W, P, B, s);     // d_v
   for (int l = L - 1; l >= 0; --l) {
+    // dv: the gradient at the layer's output; in the fused path already at its z
     const float* dz = f->dv;
-    if (l < L - 1) {
+    const bool fused = fused_size(f, N);
+    if (l < L - 1 && !fused) {
       k_gelu_bwd<<<blocks_for(bc * P), FT, 0, s>>>(f->dv, f->z[l], f->dz, bc * P);
       note_launches(1);
       dz = f->dz;
     }
     wgrad(dz, W, f->v[l], W, f->g + f->o_Ww + (size_t)l * W * W, f->g + f->o_Wb + (size_t)l * W, f->part, P, B, s);
-    // pointwise branch of d_vin into dt
-    pw<true, false, false>(dz, W, f->wb + f->o_Ww + (size_t)l * W * W, nullptr, f->dt, nullptr, W, P, B, s);
     // spectral branch: dY = (c/N^2) dft(dz); dR = sum_b conj(Xh) dY; dXh = sum_o conj(R) dY
     dft_y(f, dz, bc * N, N, s);
     // (and d_vin += Re(sum dXh e^{+i theta}), the adjoint of the forward transform)
     modes_x<true>(f, l, f->dY, f->cky_s, B, N, s);
     k_mix_wgrad<<<blocks_for((size_t)W * W * nm), FT, 0, s>>>(f->Xh[l], f->dY, f->g + f->o_Rre + (size_t)l * W * W * nm,
                                                           f->g + f->o_Rim + (size_t)l * W * W * nm, W, (int)nm, B);
+    if (fused) {
+      layer_fused_bwd(f, l, dz, l > 0 ? f->z[l - 1] : nullptr, f->dt, B, N, s);
+      note_launches(2);
+      std::swap(f->dv, f->dt);
+      continue;
+    }
+    // pointwise branch of d_vin into dt
+    pw<true, false, false>(dz, W, f->wb + f->o_Ww + (size_t)l * W * W, nullptr, f->dt, nullptr, W, P, B, s);
     idft_y<true>(f, f->dt, nullptr, 1.f, bc * N, N, s);
     note_launches(3);
     std::swap(f->dv, f->dt);
   }
   wgrad(f->dv, W, x, 7, f->g + f->o_Pw, f->g + f->o_Pb, f->part, P, B, s);
   BEM_CUDA_TRY(cudaGetLastError());
+  // (a copy to pageable memory waits for the stream: after everything is launched)
+  std::vector<double> lp(lb);
+  BEM_CUDA_TRY(cudaMemcpyAsync(lp.data(), f->lpart, lb * sizeof(double), cudaMemcpyDeviceToHost, s));
   BEM_CUDA_TRY(cudaStreamSynchronize(s));
   double sum = 0.0;
   for (double v : lp) sum += v;
