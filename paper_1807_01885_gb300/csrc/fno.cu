@@ -545,6 +545,7 @@ __global__ void __launch_bounds__(128) k_pw_tc(const float* __restrict__ X, int 
 }
 
 #include "fno_grad.cuh"
+#include "fno_proj.cuh"
 
 // ---- fused Fourier layer (forward) --------------------------------------------
 // One kernel for z = W v + b + S(v) and v' = gelu(z): for 16 pixels y of one row x of
@@ -1301,7 +1302,7 @@ struct bem_fno_s {
   std::vector<float*> v, z;
   std::vector<float2*> Xh;
   float *a = nullptr, *h = nullptr, *out = nullptr, *dout = nullptr;
-  float *dv = nullptr, *dz = nullptr, *dt = nullptr, *mom = nullptr, *part = nullptr, *cky = nullptr, *cky_s = nullptr;
+  float *dv = nullptr, *dz = nullptr, *dt = nullptr, *mom = nullptr, *part = nullptr, *part2 = nullptr, *cky = nullptr, *cky_s = nullptr;
   double* mom_part = nullptr;   // per-chunk sums of the height moments
   float2 *A = nullptr, *Y = nullptr, *dY = nullptr, *Xp = nullptr, *tw = nullptr, *twx = nullptr;
   float *Tf = nullptr, *Ti = nullptr;   // twiddle matrices of the y transforms (N x 2m, 2m x N)
@@ -1328,8 +1329,11 @@ bool fused_ok(const bem_fno_s* f) {
   const int W = f->d.width;
   return tc_ok(f) && (W == 8 || W == 16 || W == 32);
 }
-// the fused projection: input width <= 32, hidden width <= 64
-bool proj_ok(const bem_fno_s* f) { return f->d.width <= 32 && f->d.hidden <= 64; }
+// the fused projection, forward and backward: input width <= 32, hidden width <= 64,
+// 32-bit offsets within a sample
+bool proj_ok(const bem_fno_s* f, int N) {
+  return f->d.width <= 32 && f->d.hidden <= 64 && (size_t)f->d.width * N * N < (size_t(1) << 32);
+}
 
 constexpr int kMaxSamples = 4096;
 // frees the activation buffers: everything allocated after the handle's persistent
@@ -1383,11 +1387,12 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
   for (int i = 0; i < nv && e == cudaSuccess; ++i) e = alloc(f, &f->v[i], (size_t)B * W * P);
   for (int i = 0; i < nz && e == cudaSuccess; ++i) e = alloc(f, &f->z[i], (size_t)B * W * P);
   for (size_t i = 0; i < f->Xh.size() && e == cudaSuccess; ++i) e = alloc(f, &f->Xh[i], (size_t)B * W * nm);
-  if (e == cudaSuccess) e = alloc(f, &f->a, (size_t)B * H * P);
-  if (e == cudaSuccess) e = alloc(f, &f->h, (size_t)B * H * P);
+  const bool hidden = !proj_ok(f, N);   // the hidden layer is stored
+  if (e == cudaSuccess && hidden) e = alloc(f, &f->a, (size_t)B * H * P);
+  if (e == cudaSuccess && hidden) e = alloc(f, &f->h, (size_t)B * H * P);
   if (e == cudaSuccess) e = alloc(f, &f->out, (size_t)B * P);
   if (e == cudaSuccess) e = alloc(f, &f->dout, (size_t)B * P);
-  const size_t big = (size_t)B * std::max(W, H) * P;
+  const size_t big = (size_t)B * (hidden ? std::max(W, H) : W) * P;
   if (e == cudaSuccess && train) e = alloc(f, &f->dv, big);
   if (e == cudaSuccess && train) e = alloc(f, &f->dz, big);
   if (e == cudaSuccess && train) e = alloc(f, &f->dt, big);
@@ -1407,6 +1412,7 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
     e = alloc(f, &f->TfA, (size_t)((N + 15) / 16) * ((2 * m + 15) / 16) * 64);
   const size_t maxout = (size_t)std::max(W, H) * std::max({W, H, 7}) + std::max(W, H);
   if (e == cudaSuccess && train) e = alloc(f, &f->part, kWgBlocks * maxout);
+  if (e == cudaSuccess && train) e = alloc(f, &f->part2, (size_t)kProjBlocks * (H + 1));
   if (e == cudaSuccess) e = alloc(f, &f->lpart, (size_t)4096);
   if (e == cudaSuccess) e = alloc(f, &f->cky, (size_t)m);
   if (e == cudaSuccess) e = alloc(f, &f->cky_s, (size_t)m);
@@ -1613,6 +1619,32 @@ void layer_fused_bwd(bem_fno_s* f, int l, const float* dz, float* zprev, float* 
   note_launches(1);
 }
 
+template <int KT, int MH>
+void proj_bwd_launch(bem_fno_s* f, const float* v, float* dv, int B, int N, cudaStream_t s) {
+  const int W = f->d.width, H = f->d.hidden;
+  const unsigned P = (unsigned)N * (unsigned)N, tps = (P + 15) / 16, tiles = tps * (unsigned)B;
+  const int nblk = (int)std::min<unsigned>(kProjBlocks, (tiles + 3) / 4);
+  k_proj_bwd<KT, MH><<<nblk, 128, 0, s>>>(v, f->dout, f->wb + f->o_Q1w, f->wb + f->o_Q1b, f->wb + f->o_Q2w, dv, f->part,
+                                          f->part2, W, H, P, tps, tiles);
+  const int n1 = H * W + H;
+  k_pw_wgrad_sum<<<(n1 + 31) / 32, 256, 0, s>>>(f->part, nblk, H * W, n1, f->g + f->o_Q1w, f->g + f->o_Q1b);
+  k_pw_wgrad_sum<<<(H + 32) / 32, 256, 0, s>>>(f->part2, nblk, H, H + 1, f->g + f->o_Q2w, f->g + f->o_Q2b);
+  note_launches(3);
+}
+
+template <int KT>
+void proj_bwd_mh(bem_fno_s* f, const float* v, float* dv, int B, int N, cudaStream_t s) {
+  if (f->d.hidden <= 16) proj_bwd_launch<KT, 1>(f, v, dv, B, N, s);
+  else if (f->d.hidden <= 32) proj_bwd_launch<KT, 2>(f, v, dv, B, N, s);
+  else proj_bwd_launch<KT, 4>(f, v, dv, B, N, s);
+}
+
+// dv and the gradients of Q1, q1, Q2, q2 from v and dout (proj_ok)
+void proj_bwd(bem_fno_s* f, const float* v, float* dv, int B, int N, cudaStream_t s) {
+  if (f->d.width <= 16) proj_bwd_mh<1>(f, v, dv, B, N, s);
+  else proj_bwd_mh<2>(f, v, dv, B, N, s);
+}
+
 bool fused_size(const bem_fno_s* f, int N) {   // 32-bit offsets within a sample
   return fused_ok(f) && (size_t)f->d.width * N * N < (size_t(1) << 32);
 }
@@ -1636,7 +1668,7 @@ void proj_nt(bem_fno_s* f, const float* v, int B, int N, cudaStream_t s) {
   else proj_launch<KT, 8>(f, v, B, N, s);
 }
 
-// out = Q2 gelu(Q1 v + q1) + q2 without storing the hidden layer (inference, proj_ok)
+// out = Q2 gelu(Q1 v + q1) + q2 without storing the hidden layer (proj_ok)
 void proj_fused(bem_fno_s* f, const float* v, int B, int N, cudaStream_t s) {
   if (f->d.width <= 16) proj_nt<1>(f, v, B, N, s);
   else proj_nt<2>(f, v, B, N, s);
@@ -1668,7 +1700,7 @@ bem_status forward(bem_fno_s* f, int B, int N, const float* x, bool train, cudaS
     }
   }
   float* vL = train ? f->v[L] : f->v[L & 1];
-  if (!train && proj_ok(f) && (size_t)W * P < (size_t(1) << 32)) {
+  if (proj_ok(f, N)) {
     proj_fused(f, vL, B, N, s);
   } else {
     pw<false, false, true>(vL, W, f->wb + f->o_Q1w, f->wb + f->o_Q1b, f->a, f->h, H, P, B, s);
@@ -1684,13 +1716,16 @@ bem_status backward(bem_fno_s* f, int B, int N, const float* x, const float* tar
   const int lb = std::min(blocks_for((size_t)B * P), 4096);
   k_mse<<<lb, FT, 0, s>>>(f->out, target, f->dout, f->lpart, (size_t)B * P);
   note_launches(1);
-  // projection
-  wgrad(f->dout, 1, f->h, H, f->g + f->o_Q2w, f->g + f->o_Q2b, f->part, P, B, s);
-  pw<true, false, false>(f->dout, 1, f->wb + f->o_Q2w, nullptr, f->dt, nullptr, H, P, B, s);   // d_h
-  k_gelu_bwd<<<blocks_for((size_t)B * H * P), FT, 0, s>>>(f->dt, f->a, f->dz, (size_t)B * H * P);   // d_a
-  note_launches(1);
-  wgrad(f->dz, H, f->v[L], W, f->g + f->o_Q1w, f->g + f->o_Q1b, f->part, P, B, s);
-  pw<true, false, false>(f->dz, H, f->wb + f->o_Q1w, nullptr, f->dv, nullptr, W, P, B, s);     // d_v
+  if (proj_ok(f, N)) {
+    proj_bwd(f, f->v[L], f->dv, B, N, s);
+  } else {
+    wgrad(f->dout, 1, f->h, H, f->g + f->o_Q2w, f->g + f->o_Q2b, f->part, P, B, s);
+    pw<true, false, false>(f->dout, 1, f->wb + f->o_Q2w, nullptr, f->dt, nullptr, H, P, B, s);   // d_h
+    k_gelu_bwd<<<blocks_for((size_t)B * H * P), FT, 0, s>>>(f->dt, f->a, f->dz, (size_t)B * H * P);   // d_a
+    note_launches(1);
+    wgrad(f->dz, H, f->v[L], W, f->g + f->o_Q1w, f->g + f->o_Q1b, f->part, P, B, s);
+    pw<true, false, false>(f->dz, H, f->wb + f->o_Q1w, nullptr, f->dv, nullptr, W, P, B, s);     // d_v
+  }
   for (int l = L - 1; l >= 0; --l) {
     // dv: the gradient at the layer's output; in the fused path already at its z
     const float* dz = f->dv;
