@@ -459,6 +459,11 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
   if (k->prec == BEM_FP32 &&
       (e = alloc_guarded(w, &w.twpc, (size_t)pair_tw_count(k->logN + 1) * 4 * sizeof(float))) != cudaSuccess)
     return fail(e, "cudaMalloc(twpc)");
+  if (k->prec == BEM_FP64 && k->logN >= 4) {
+    if ((e = alloc_guarded(w, &w.fexp, (size_t)(2 * k->N + 1) * sizeof(int))) != cudaSuccess)
+      return fail(e, "cudaMalloc(fexp)");
+    if ((e = alloc_guarded(w, &w.twf, fix_tw_bytes(k))) != cudaSuccess) return fail(e, "cudaMalloc(twf)");
+  }
   if ((e = alloc_guarded(w, &w.vec, 7 * n * k->elem)) != cudaSuccess) return fail(e, "cudaMalloc(vec)");
   if ((e = alloc_guarded(w, &w.mask, 2 * n)) != cudaSuccess) return fail(e, "cudaMalloc(mask)");
   if ((e = alloc_guarded(w, &w.partials, 16 * 2048 * sizeof(double))) != cudaSuccess)
@@ -595,9 +600,9 @@ bem_status bem_matvec(bem_kernel k, const void* p, void* u, void* cuda_stream) {
   void* ud = u_host ? k->ws.stage_out : u;
   if (((uintptr_t)ud & 15) != 0) { set_error("u must be 16-byte aligned"); return BEM_EINVAL; }
   if (k->prec == BEM_FP64)
-    launch_matvec<double>(k, (const double*)ap.dev, (double*)ud, s, nullptr);
+    launch_product<double>(k, (const double*)ap.dev, (double*)ud, s);
   else
-    launch_matvec<float>(k, (const float*)ap.dev, (float*)ud, s, nullptr);
+    launch_product<float>(k, (const float*)ap.dev, (float*)ud, s);
   BEM_CUDA_TRY(cudaGetLastError());
   if (u_host) {
     BEM_CUDA_TRY(cudaMemcpyAsync(u, ud, bytes, cudaMemcpyDeviceToHost, s));

@@ -137,6 +137,8 @@ struct Workspace {
   void* twr = nullptr;       // stage twiddles of the length-N register FFT (rows)
   void* twc = nullptr;       // stage twiddles of the length-2N register FFT (columns)
   void* twpc = nullptr;      // float path: broadcast stage twiddles of the paired column FFT (4N float4)
+  int* fexp = nullptr;       // fixed-point product (double, N >= 16): exponents of the rows and columns (2N + 1)
+  void* twf = nullptr;       // and its twiddles: M records, then the stages of lengths N and 2N
   void* vec = nullptr;       // solver vectors: p, g, t, r, u, f, x (N*N each)
   uint8_t* mask = nullptr;   // N*N contact mask (adhesive), plus a second copy; PK: contact set {p > 0}
   double* partials = nullptr;// per-block partial sums
@@ -272,7 +274,7 @@ inline bool open_plane_homogeneous(const bem_kernel_desc& d, double* E = nullptr
 bem_status build_table(bem_kernel_s* k, cudaStream_t s);
 template <typename T>
 void launch_matvec(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s, const int* skip_flag);
-// one pass of the product (0 = rows forward, 1 = columns, 2 = rows inverse)
+// one pass of bem_matvec's product (0 = rows forward, 1 = columns, 2 = rows inverse)
 template <typename T>
 void launch_pass(const bem_kernel_s* k, int pass, const T* p, T* u, cudaStream_t s);
 size_t spec_bytes(const bem_kernel_s* k);
@@ -283,6 +285,13 @@ template <typename T>
 void reg_twiddles(const bem_kernel_s* k, cudaStream_t s);
 template <typename T>
 void reg_prepare(const bem_kernel_s* k);
+// matvec_fix.cu (double, N >= 16): one pass of the fixed-point product, its twiddles
+void fix_pass(const bem_kernel_s* k, int which, const double* p, double* u, cudaStream_t s);
+void fix_twiddles(const bem_kernel_s* k, cudaStream_t s);
+size_t fix_tw_bytes(const bem_kernel_s* k);
+// matvec.cu: the product of bem_matvec; a pass of it as launch_pass does for the solves'
+template <typename T>
+void launch_product(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s);
 // matvec.cu: sets the one-time kernel attributes of the product's passes for k
 // (what the first plain launch would set), so that a graph capture can follow
 template <typename T>

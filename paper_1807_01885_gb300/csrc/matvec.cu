@@ -325,7 +325,10 @@ bem_status build_table(bem_kernel_s* k, cudaStream_t s) {
     if (k->logN >= 4) k_table_square<double><<<256, 256, 0, s>>>(k->ws.table64, (double*)k->ws.table, k->N, scale);
     else k_table_block<double><<<256, 256, 0, s>>>(k->ws.table64, (double*)k->ws.table, k->N, scale);
     k_twiddles<double><<<(k->M + 255) / 256, 256, 0, s>>>((double2*)k->ws.tw, k->M);
-    if (k->logN >= 4) reg_twiddles<double>(k, s);
+    if (k->logN >= 4) {
+      reg_twiddles<double>(k, s);
+      fix_twiddles(k, s);
+    }
   } else {
     if (k->logN >= 4) k_table_pair<<<256, 256, 0, s>>>(k->ws.table64, (float2*)k->ws.table, k->N, scale);
     else k_table_block<float><<<256, 256, 0, s>>>(k->ws.table64, (float*)k->ws.table, k->N, scale);
@@ -519,24 +522,42 @@ void harvest_pass_timing(const bem_kernel_s* k) {
   }
 }
 
-template <typename T>
-void launch_matvec(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s, const int* skip) {
-  for (int pass = 0; pass < 3; ++pass) {
+// the three passes on s, with events around each while pass timing is on
+template <typename F>
+static void run_passes(const bem_kernel_s* k, cudaStream_t s, F&& pass) {
+  for (int i = 0; i < 3; ++i) {
     if (k->timing.on) {
       auto e = timing_pair(k);
       cudaEventRecord(e.first, s);
-      pass_impl<T>(k, pass, p, u, s, skip);
+      pass(i);
       cudaEventRecord(e.second, s);
-      k->timing.pending[pass].push_back(e);
+      k->timing.pending[i].push_back(e);
     } else {
-      pass_impl<T>(k, pass, p, u, s, skip);
+      pass(i);
     }
   }
 }
 
 template <typename T>
+void launch_matvec(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s, const int* skip) {
+  run_passes(k, s, [&](int pass) { pass_impl<T>(k, pass, p, u, s, skip); });
+}
+
+template <typename T>
 void launch_pass(const bem_kernel_s* k, int pass, const T* p, T* u, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (k->logN >= 4) {
+      fix_pass(k, pass, p, u, s);
+      note_launches(1);
+      return;
+    }
+  }
   pass_impl<T>(k, pass, p, u, s, nullptr);
+}
+
+template <typename T>
+void launch_product(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s) {
+  run_passes(k, s, [&](int pass) { launch_pass<T>(k, pass, p, u, s); });
 }
 
 template <typename T>
@@ -547,6 +568,8 @@ void prepare_passes(const bem_kernel_s* k) {
 
 template void prepare_passes<float>(const bem_kernel_s*);
 template void prepare_passes<double>(const bem_kernel_s*);
+template void launch_product<float>(const bem_kernel_s*, const float*, float*, cudaStream_t);
+template void launch_product<double>(const bem_kernel_s*, const double*, double*, cudaStream_t);
 template void launch_pass<float>(const bem_kernel_s*, int, const float*, float*, cudaStream_t);
 template void launch_pass<double>(const bem_kernel_s*, int, const double*, double*, cudaStream_t);
 template void launch_matvec<float>(const bem_kernel_s*, const float*, float*, cudaStream_t, const int*);
