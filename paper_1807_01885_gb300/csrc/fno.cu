@@ -1539,7 +1539,7 @@ void modes_x(bem_fno_s* f, int l, float2* Xh, const float* wky, int B, int N, cu
   const bf16* Rre = f->wb + f->o_Rre + (size_t)l * W * W * nm;
   const bf16* Rim = f->wb + f->o_Rim + (size_t)l * W * W * nm;
   const bool tiled = m <= kXModes;
-  const int chunks = tiled ? dft_x_chunks(bc, N) : 1;
+  const int chunks = tiled ? dft_x_chunks(bc, N, m) : 1;
   float2* Xp = chunks > 1 ? f->Xp : Xh;
   if (tiled) k_dft_x<<<dim3((unsigned)bc, chunks), 256, 0, s>>>(f->A, Xp, f->twx, wky, N, m);
   else k_dft_x_any<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, Xp, f->tw, wky, N, m);

@@ -14,7 +14,10 @@
 // of N = 256, m = 16; twiddles gathered by every block 28 and 20 us.)
 #pragma once
 
-constexpr int kXRows = 64;        // rows x staged in shared memory at a time
+constexpr int kXRows = 64;        // rows x per block of the inverse
+// rows x that the forward transform stages at a time: few modes leave room for more, and
+// their many slices want them (m = 4 with 64 rows was no faster than the gathered form)
+__host__ __device__ inline int dft_x_rows(int m) { return m <= 4 ? 256 : (m <= 12 ? 128 : 64); }
 constexpr int kXModes = 32;       // most modes per axis that the tiled kernels take
 constexpr int kXBlocks = 912;     // blocks that fill the GPU (six per SM)
 
@@ -31,8 +34,8 @@ __global__ void k_twiddle_x(const float2* __restrict__ tw, float2* __restrict__ 
 }
 
 // blocks per channel along x of k_dft_x (each adds its share of the rows)
-inline int dft_x_chunks(size_t bc, int N) {
-  const size_t tiles = (N + kXRows - 1) / kXRows, want = (kXBlocks + bc - 1) / bc;
+inline int dft_x_chunks(size_t bc, int N, int m) {
+  const size_t tiles = (N + dft_x_rows(m) - 1) / dft_x_rows(m), want = (kXBlocks + bc - 1) / bc;
   return (int)std::min(tiles, std::max<size_t>(want, 1));
 }
 
@@ -40,19 +43,20 @@ inline int dft_x_chunks(size_t bc, int N) {
 __global__ void __launch_bounds__(256) k_dft_x(const float2* __restrict__ A, float2* __restrict__ Xp,
                                                const float2* __restrict__ twx, const float* __restrict__ wky, int N,
                                                int m) {
-  __shared__ __align__(16) float smem[kXRows * (kXModes * 2 + 36 * 2)];
+  __shared__ __align__(16) float smem[64 * (kXModes * 2 + 36 * 2)];   // rows (2 ky2 + kt) float2 at every m, and 256 x 32
+  const int rows = dft_x_rows(m);
   const int ky2 = (m + 1) / 2, kg = (m + 4) / 4, kt = dft_x_kt(m), items = ky2 * kg, S = 256 / items;
-  float2* const sA = reinterpret_cast<float2*>(smem);                  // [kXRows][2 ky2]
-  float2* const sT = sA + kXRows * 2 * ky2;                            // [kXRows][kt]
+  float2* const sA = reinterpret_cast<float2*>(smem);                  // [rows][2 ky2]
+  float2* const sT = sA + rows * 2 * ky2;                              // [rows][kt]
   const size_t q = blockIdx.x;
   const int tid = threadIdx.x, slice = tid / items, item = tid - slice * items;
   const int kyp = item % ky2, k0 = 4 * (item / ky2);
-  const int tiles = (N + kXRows - 1) / kXRows;
+  const int tiles = (N + rows - 1) / rows;
   const int t0 = (int)((long long)tiles * blockIdx.y / gridDim.y), t1 = (int)((long long)tiles * (blockIdx.y + 1) / gridDim.y);
   // sums of re wx, im wy, re wy, im wx for 4 k and 2 ky
   float acc[4][2][4] = {};
   for (int tile = t0; tile < t1; ++tile) {
-    const int x0 = tile * kXRows, nx = min(kXRows, N - x0);
+    const int x0 = tile * rows, nx = min(rows, N - x0);
     __syncthreads();
     if (m % 2 == 0) {
       const float4* a = reinterpret_cast<const float4*>(A + (q * N + x0) * m);
@@ -98,18 +102,21 @@ __global__ void __launch_bounds__(256) k_dft_x(const float2* __restrict__ A, flo
         for (int e = 0; e < 4; ++e) red[(slice * 32 + (k * 2 + h) * 4 + e) * items + item] = acc[k][h][e];
   }
   __syncthreads();
+  for (int o = tid; o < items * 32; o += 256) {
+    float s = red[o];
+    for (int sl = 1; sl < S; ++sl) s += red[sl * 32 * items + o];
+    red[o] = s;
+  }
+  __syncthreads();
   float2* out = Xp + ((size_t)blockIdx.y * gridDim.x + q) * 2 * m * m;
   for (int o = tid; o < items * 8; o += 256) {
     const int it = o % items, kh = o / items;
     const int k = 4 * (it / ky2) + kh / 2, ky = 2 * (it % ky2) + (kh & 1);
     if (k > m || ky >= m) continue;
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int sl = 0; sl < S; ++sl)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) s[e] += red[(sl * 32 + kh * 4 + e) * items + it];
+    const float* s = red + kh * 4 * items + it;
     const float sc = wky != nullptr ? wky[ky] : 1.f;
-    if (k < m) out[k * m + ky] = make_float2((s[0] - s[1]) * sc, (s[2] + s[3]) * sc);
-    if (k > 0) out[(2 * m - k) * m + ky] = make_float2((s[0] + s[1]) * sc, (s[3] - s[2]) * sc);
+    if (k < m) out[k * m + ky] = make_float2((s[0] - s[items]) * sc, (s[2 * items] + s[3 * items]) * sc);
+    if (k > 0) out[(2 * m - k) * m + ky] = make_float2((s[0] + s[items]) * sc, (s[3 * items] - s[2 * items]) * sc);
   }
 }
 
