@@ -465,7 +465,7 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
     if ((e = alloc_guarded(w, &w.twf, fix_tw_bytes(k))) != cudaSuccess) return fail(e, "cudaMalloc(twf)");
   }
   if ((e = alloc_guarded(w, &w.vec, 7 * n * k->elem)) != cudaSuccess) return fail(e, "cudaMalloc(vec)");
-  if ((e = alloc_guarded(w, &w.mask, 2 * n)) != cudaSuccess) return fail(e, "cudaMalloc(mask)");
+  if ((e = alloc_guarded(w, &w.mask, 2 * n + n / 4)) != cudaSuccess) return fail(e, "cudaMalloc(mask)");
   if ((e = alloc_guarded(w, &w.partials, 16 * 2048 * sizeof(double))) != cudaSuccess)
     return fail(e, "cudaMalloc(partials)");
   if ((e = cudaMalloc((void**)&w.ticket, sizeof(unsigned int))) != cudaSuccess) return fail(e, "cudaMalloc(ticket)");

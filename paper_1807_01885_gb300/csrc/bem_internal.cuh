@@ -140,7 +140,7 @@ struct Workspace {
   int* fexp = nullptr;       // fixed-point product (double, N >= 16): exponents of the rows and columns (2N + 1)
   void* twf = nullptr;       // and its twiddles: M records, then the stages of lengths N and 2N
   void* vec = nullptr;       // solver vectors: p, g, t, r, u, f, x (N*N each)
-  uint8_t* mask = nullptr;   // N*N contact mask (adhesive), plus a second copy; PK: contact set {p > 0}
+  uint8_t* mask = nullptr;   // N*N contact mask (adhesive), plus a second copy; PK: two contact sets, N*N/4 change flags
   double* partials = nullptr;// per-block partial sums
   unsigned int* ticket = nullptr;
   SolveState* state = nullptr;

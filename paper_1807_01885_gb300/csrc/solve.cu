@@ -57,6 +57,17 @@ int red_blocks(size_t n, int per_sm) {
   b = std::max<size_t>(1, std::min<size_t>(b, RED_MAX_BLOCKS));
   return (int)b;
 }
+// The same for the adhesive CG, which runs alone on the GPU: in float up to 256 blocks with
+// one group of four elements per thread, so that the sweep of a middle grid is one round
+// of loads (N = 512 on 64 blocks: adhesive ramp 30.3 ms, on 256: 25.8).  The constrained
+// CG keeps sixteen elements per thread, because many of its solves run side by side (a
+// batch of 32 at N = 256: 6.5 ms, with 64 blocks 7.2), and so does double, where another
+// grouping is another order of the sums: a solve of a symmetric problem follows their
+// last place and would return other pressures at the level of its tolerance.
+int lin_blocks(size_t n, size_t elem) {
+  const size_t b = (size_t)red_blocks(n, 4);
+  return elem == 4 ? (int)std::max(b, std::min<size_t>(256, (n + NTHREADS * 4 - 1) / (NTHREADS * 4))) : (int)b;
+}
 
 #define GRID_STRIDE(i, n) \
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (n); i += (size_t)gridDim.x * blockDim.x)
@@ -93,20 +104,31 @@ __device__ __forceinline__ void finish(SolveState* st, int status) {
 
 // Initial guess for depth control: q = max(d - f, 0) scaled by the energy-optimal
 // factor s = <q, d - f> / <q, K q>; the gap then follows from u = K q as s u + f - d.
-// contact-set bytes of four consecutive cells: (p > 0) written by k_pk_begin, read
-// by the sweeps that need only the set (p keeps its sign until k_pk_update)
+// The sweeps touch what an iteration changes.  The contact set is a few per cent of the
+// cells of a rough surface and a sixth of a sphere's or a punch's window; outside it p and
+// t are zero and stay so, and the pending changes x are zero but for a few cells.  The set
+// is kept as one byte per cell (p > 0), written by k_pk_update for the next iteration in
+// the other of two buffers (the previous set tells where t must be cleared), and xm holds
+// one byte per group of four cells whose x may not be zero.  Groups of four cells without
+// a contact cell then cost their byte word (and, where the gap itself moves, the gap's
+// arrays): 340 -> 150 MB per iteration at N = 2048, and in double the arithmetic of the
+// sums, which bounds those sweeps.  The sums only lose zeros: results are unchanged.
+// Measured on GB300: @SW@.
 template <typename T>
 __device__ __forceinline__ void stm4(uint8_t* m, size_t i4, const T (&pv)[4]) {
   reinterpret_cast<uchar4*>(m)[i4] =
       make_uchar4(pv[0] > (T)0, pv[1] > (T)0, pv[2] > (T)0, pv[3] > (T)0);
 }
-__device__ __forceinline__ void ldm4(const uint8_t* m, size_t i4, bool (&o)[4]) {
-  const uchar4 v = reinterpret_cast<const uchar4*>(m)[i4];
-  o[0] = v.x != 0;
-  o[1] = v.y != 0;
-  o[2] = v.z != 0;
-  o[3] = v.w != 0;
+// returns whether any of the four is in the set
+__device__ __forceinline__ bool ldm4(const uint8_t* m, size_t i4, bool (&o)[4]) {
+  const unsigned v = reinterpret_cast<const unsigned*>(m)[i4];
+  o[0] = (v & 0xffu) != 0;
+  o[1] = (v & 0xff00u) != 0;
+  o[2] = (v & 0xff0000u) != 0;
+  o[3] = (v & 0xff000000u) != 0;
+  return v != 0u;
 }
+__device__ __forceinline__ bool anym4(const uint8_t* m, size_t i4) { return reinterpret_cast<const unsigned*>(m)[i4] != 0u; }
 
 template <typename T>
 __global__ void k_init_q(const T* __restrict__ f, T* __restrict__ q, double d, size_t n) {
@@ -180,8 +202,8 @@ __global__ void k_init_gap(const T* __restrict__ f, const T* __restrict__ p, T* 
 // and the set itself as bytes for the sweeps up to the update.
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T* __restrict__ p, T* __restrict__ g, const T* __restrict__ f, T* __restrict__ dp,
-                           const T* __restrict__ u, uint8_t* __restrict__ cm, double* partials,
-                           unsigned int* ticket, SolveState* st, size_t n) {
+                           const T* __restrict__ u, const uint8_t* __restrict__ cm, const uint8_t* __restrict__ xm,
+                           double* partials, unsigned int* ticket, SolveState* st, size_t n) {
   pdl_enter();
   if (st->done) return;
   const double s = st->scale, d = st->d;
@@ -193,33 +215,39 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T
   Acc<T> ag, agg, auu, ap, cnt;
   VEC_LOOP(i4, n) {
     T pv[4], gv[4], fv[4];
-    ld4(p, i4, pv);
+    const bool any = anym4(cm, i4);
+    if (!any && !refresh && !apply) continue;
     ld4(g, i4, gv);
-    ld4(f, i4, fv);
+    if (any || s1 != (T)0) ld4(f, i4, fv);
+    if (any) ld4(p, i4, pv);
     if (refresh) {
       T uv[4];
       ld4(u, i4, uv);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        gv[e] = sT * (gv[e] + uv[e]) + s1 * (dT - fv[e]);
-        pv[e] = sT * pv[e];
+        if (any || s1 != (T)0) gv[e] = sT * (gv[e] + uv[e]) + s1 * (dT - fv[e]);
+        else gv[e] = gv[e] + uv[e];      // scale 1
+        if (any) pv[e] = sT * pv[e];
       }
-      st4(p, i4, pv);
+      if (any) st4(p, i4, pv);
       st4(g, i4, gv);
     } else if (apply) {
-      T xv[4];
-      ld4(dp, i4, xv);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        pv[e] = sT * pv[e];
-        gv[e] = sT * gv[e] + s1 * (dT - fv[e]);
-        xv[e] = sT * xv[e];     // pending changes scale with p
+        if (any) pv[e] = sT * pv[e];
+        if (any || s1 != (T)0) gv[e] = sT * gv[e] + s1 * (dT - fv[e]);
       }
-      st4(p, i4, pv);
+      if (any) st4(p, i4, pv);
       st4(g, i4, gv);
-      st4(dp, i4, xv);
+      if (xm[i4]) {
+        T xv[4];
+        ld4(dp, i4, xv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xv[e] = sT * xv[e];     // pending changes scale with p
+        st4(dp, i4, xv);
+      }
     }
-    stm4(cm, i4, pv);
+    if (!any) continue;
     T sg[4], suu[4], sp[4], sc[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -233,12 +261,10 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T
     // the gap sums element by element, with exact squares: under force control G is
     // their difference sum g^2 - 2 gbar sum g + n gbar^2, which cancels when the gaps
     // share a large common offset (a depth far off after a replacement, say)
-    if (sc[0] + sc[1] + sc[2] + sc[3] > (T)0) {   // groups without a contact cell add nothing
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        ag.add(sg[e]);
-        agg.add_sq(sg[e]);
-      }
+    for (int e = 0; e < 4; ++e) {
+      ag.add(sg[e]);
+      agg.add_sq(sg[e]);
     }
     auu.add4(suu);
     ap.add4(sp);
@@ -302,15 +328,22 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T
 // The shifted gap g - gbar is not stored: k_pk_rt and k_pk_update form the same
 // float value from g when they read it, and k_pk_update stores the shifted step.
 template <typename T>
-__global__ void k_pk_dir(const uint8_t* __restrict__ cm, const T* __restrict__ g, T* __restrict__ t,
-                         const SolveState* st, size_t n) {
+__global__ void k_pk_dir(const uint8_t* __restrict__ cm, const uint8_t* __restrict__ cm_prev, const T* __restrict__ g,
+                         T* __restrict__ t, const SolveState* st, size_t n) {
   pdl_enter();
   if (st->done) return;
   const T gbar = (T)st->gbar, beta = (T)st->beta;
   VEC_LOOP(i4, n) {
     T gv[4], tv[4];
     bool in[4];
-    ldm4(cm, i4, in);
+    const bool prev = anym4(cm_prev, i4);
+    if (!ldm4(cm, i4, in)) {
+      if (prev) {
+        const T zero[4] = {(T)0, (T)0, (T)0, (T)0};
+        st4(t, i4, zero);
+      }
+      continue;
+    }
     ld4(g, i4, gv);
     ld4(t, i4, tv);
 #pragma unroll
@@ -330,7 +363,7 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 6 : 1) k_pk_rt(cons
   VEC_LOOP(i4, n) {
     T gv[4], tv[4], rv[4];
     bool in[4];
-    ldm4(cm, i4, in);
+    if (!ldm4(cm, i4, in)) continue;
     ld4(g, i4, gv);
     ld4(t, i4, tv);
     ld4(r, i4, rv);
@@ -392,8 +425,9 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 6 : 1) k_pk_rt(cons
 // that the next correction computes g = K p + f - d from scratch.
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_update(T* __restrict__ p, T* __restrict__ g, const T* __restrict__ t, const T* __restrict__ r,
-                            T* __restrict__ dp, const T* __restrict__ f, double* partials, unsigned int* ticket,
-                            SolveState* st, size_t n) {
+                            T* __restrict__ dp, const T* __restrict__ f, const uint8_t* __restrict__ cm,
+                            uint8_t* __restrict__ cm_next, uint8_t* __restrict__ xm, double* partials,
+                            unsigned int* ticket, SolveState* st, size_t n) {
   pdl_enter();
   if (st->done) return;
   const T tau = (T)st->tau;
@@ -408,52 +442,69 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_update(
   const T gthr = -noise * (T)st->uscale, pthr = -noise * (T)st->pscale;
   Acc<T> asum, nneg, nol;
   VEC_LOOP(i4, n) {
-    T pv[4], gv[4], tv[4], rv[4], dv[4] = {(T)0, (T)0, (T)0, (T)0};
-    ld4(p, i4, pv);
+    T pv[4] = {(T)0, (T)0, (T)0, (T)0}, tv[4], gv[4], rv[4], ch[4] = {(T)0, (T)0, (T)0, (T)0};
+    const bool any = anym4(cm, i4);
+    const bool xold = xm[i4] != 0;
     ld4(g, i4, gv);
-    ld4(t, i4, tv);
     ld4(r, i4, rv);
-    if (!xz) ld4(dp, i4, dv);
+    if (any) {
+      ld4(p, i4, pv);
+      ld4(t, i4, tv);
+    }
     T cneg[4], col[4];
+    bool touched = any, changed = false;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const T pi = pv[e], gi = gv[e] - gbar;
-      T pn, dpn = dv[e];      // changes not yet applied to g accumulate until the next correction
+      T pn;
       cneg[e] = (T)0;
       col[e] = (T)0;
       if (pi > (T)0) {
         pn = pi - tau * tv[e];
         if (pn < (T)0) {
           if (pn < pthr) cneg[e] = (T)1;
-          dpn -= pn;          // the projection moves p from pn to 0
+          ch[e] = -pn;          // the projection moves p from pn to 0
+          changed = true;
           pn = (T)0;
         }
       } else if (gi < gthr) {
         pn = -tau * gi;
-        dpn += pn;            // re-activation: p moves from 0 to pn
+        ch[e] = pn;             // re-activation: p moves from 0 to pn
+        changed = true;
+        touched = true;
         col[e] = (T)1;
       } else {
         pn = (T)0;
       }
       pv[e] = pn;
-      dv[e] = dpn;
       gv[e] = gi - tau * rv[e];
     }
-    asum.add4(pv);
-    nneg.add4(cneg);
-    nol.add4(col);
+    if (touched) {
+      asum.add4(pv);
+      nneg.add4(cneg);
+      nol.add4(col);
+      st4(p, i4, pv);
+    }
+    stm4(cm_next, i4, pv);
     if (replace) {
       T fv[4];
       ld4(f, i4, fv);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        dv[e] = pv[e];
-        gv[e] = fv[e] - dT;
+      for (int e = 0; e < 4; ++e) gv[e] = fv[e] - dT;
+      if (touched || xold) {
+        st4(dp, i4, pv);
+        xm[i4] = touched ? 1 : 0;
       }
+    } else if (changed || (xz && xold)) {
+      // changes not yet applied to g accumulate until the next correction
+      T dv[4] = {(T)0, (T)0, (T)0, (T)0};
+      if (!xz && xold) ld4(dp, i4, dv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dv[e] += ch[e];
+      st4(dp, i4, dv);
+      xm[i4] = changed || (xold && !xz) ? 1 : 0;
     }
-    st4(p, i4, pv);
     st4(g, i4, gv);
-    st4(dp, i4, dv);
   }
   Acc<T> v[3] = {asum, nneg, nol};
   double tot[3];
@@ -558,11 +609,35 @@ __global__ void k_lin_alpha(const T* __restrict__ s, const T* __restrict__ q, co
   if (st->done) return;
   const bool force = st->control == BEM_CTRL_FORCE;
   Acc<T> a, aq, ar;
-  GRID_STRIDE(i, n) if (C[i]) {
-    a.add(s[i] * q[i]);
-    if (force) {
-      aq.add(q[i]);
-      ar.add(r[i]);
+  if constexpr (sizeof(T) == 4) {
+    VEC_LOOP(i4, n) {
+      bool in[4];
+      T sv[4], qv[4], p4[4];
+      if (!ldm4(C, i4, in)) continue;
+      ld4(s, i4, sv);
+      ld4(q, i4, qv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) p4[e] = in[e] ? sv[e] * qv[e] : (T)0;
+      a.add4(p4);
+      if (force) {
+        T rv[4];
+        ld4(r, i4, rv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          qv[e] = in[e] ? qv[e] : (T)0;
+          rv[e] = in[e] ? rv[e] : (T)0;
+        }
+        aq.add4(qv);
+        ar.add4(rv);
+      }
+    }
+  } else {
+    GRID_STRIDE(i, n) if (C[i]) {
+      a.add(s[i] * q[i]);
+      if (force) {
+        aq.add(q[i]);
+        ar.add(r[i]);
+      }
     }
   }
   Acc<T> v[3] = {a, aq, ar};
@@ -588,12 +663,35 @@ __global__ void k_lin_update(T* __restrict__ x, T* __restrict__ r, const T* __re
   const T alpha = (T)st->alpha;
   const T qbar = (T)st->qbar, rbar = (T)st->lin_rbar;   // 0 under depth control
   Acc<T> arr;
-  GRID_STRIDE(i, n) {
-    if (C[i]) {
-      x[i] += alpha * s[i];
-      const T ri = (r[i] - rbar) - alpha * (q[i] - qbar);
-      r[i] = ri;
-      arr.add(ri * ri);
+  if constexpr (sizeof(T) == 4) {
+    VEC_LOOP(i4, n) {
+      bool in[4];
+      T xv[4], rv[4], sv[4], qv[4], r2[4];
+      if (!ldm4(C, i4, in)) continue;
+      ld4(x, i4, xv);
+      ld4(r, i4, rv);
+      ld4(s, i4, sv);
+      ld4(q, i4, qv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (in[e]) {
+          xv[e] += alpha * sv[e];
+          rv[e] = (rv[e] - rbar) - alpha * (qv[e] - qbar);
+        }
+        r2[e] = in[e] ? rv[e] * rv[e] : (T)0;
+      }
+      st4(x, i4, xv);
+      st4(r, i4, rv);
+      arr.add4(r2);
+    }
+  } else {
+    GRID_STRIDE(i, n) {
+      if (C[i]) {
+        x[i] += alpha * s[i];
+        const T ri = (r[i] - rbar) - alpha * (q[i] - qbar);
+        r[i] = ri;
+        arr.add(ri * ri);
+      }
     }
   }
   Acc<T> v[1] = {arr};
@@ -623,7 +721,16 @@ __global__ void k_lin_dir(const T* __restrict__ r, T* __restrict__ s, const uint
   pdl_enter();
   if (st->done) return;
   const T beta = (T)st->beta;
-  GRID_STRIDE(i, n) s[i] = C[i] ? r[i] + beta * s[i] : (T)0;
+  VEC_LOOP(i4, n) {
+    bool in[4];
+    T rv[4], sv[4];
+    if (!ldm4(C, i4, in)) continue;   // s is zero outside C (k_lin_init)
+    ld4(r, i4, rv);
+    ld4(s, i4, sv);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) sv[e] = in[e] ? rv[e] + beta * sv[e] : (T)0;
+    st4(s, i4, sv);
+  }
 }
 
 // Adhesive force control (Sec. 2 procedure at a given total force F): the fixed-area
@@ -770,7 +877,7 @@ bem_status read_state(bem_kernel_s* k, cudaStream_t s) {
 
 struct Ctx {
   size_t n;
-  int rb, rb6, eb;   // reduction blocks (4 and 6 per SM), element-wise blocks
+  int rb, rb6, rbl, eb;   // reduction blocks (4 and 6 per SM, adhesive CG), element-wise blocks
 };
 
 template <typename T>
@@ -779,6 +886,7 @@ Ctx ctx_of(const bem_kernel_s* k) {
   c.n = (size_t)k->N * k->N;
   c.rb = red_blocks(c.n, 4);
   c.rb6 = red_blocks(c.n, 6);
+  c.rbl = lin_blocks(c.n, sizeof(T));
   c.eb = (int)std::min<size_t>((c.n / 4 + NTHREADS - 1) / NTHREADS, 152 * 8);
   return c;
 }
@@ -814,6 +922,28 @@ void fill_result(const bem_kernel_s* k, const bem_problem* prob, double d, bem_s
   res->area = delta2 * n_c;
   res->a_eq = sqrt(res->area / M_PI);
   res->status = st;
+}
+
+// The constrained CG's sets in the handle's mask array (the adhesive masks are not live
+// during one): two buffers of a byte per cell, and xm, a byte per group of four cells.
+struct PkSets { uint8_t *cm[2], *xm; };
+PkSets pk_sets(const bem_kernel_s* k) {
+  const size_t n = (size_t)k->N * k->N;
+  return PkSets{{k->ws.mask, k->ws.mask + n}, k->ws.mask + 2 * n};
+}
+
+// First contact set {p > 0}, no previous one, and the groups with pending changes
+template <typename T>
+__global__ void k_init_sets(const T* __restrict__ p, const T* __restrict__ x, uint8_t* __restrict__ cm,
+                            uint8_t* __restrict__ cm_prev, uint8_t* __restrict__ xm, size_t n) {
+  VEC_LOOP(i4, n) {
+    T pv[4], xv[4];
+    ld4(p, i4, pv);
+    ld4(x, i4, xv);
+    stm4(cm, i4, pv);
+    reinterpret_cast<unsigned*>(cm_prev)[i4] = 0u;
+    xm[i4] = xv[0] != (T)0 || xv[1] != (T)0 || xv[2] != (T)0 || xv[3] != (T)0 ? 1 : 0;
+  }
 }
 
 // Initial state and first iterate of the Polonsky-Keer solve (asynchronous on s).
@@ -872,6 +1002,9 @@ bem_status pk_setup(bem_kernel_s* k, const bem_problem* prob, const T* pinit, cu
     k_init_apply<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.x, v.u, v.p, v.g, st, c.n);
     note_launches(1);
   }
+  const PkSets m = pk_sets(k);
+  k_init_sets<T><<<c.eb, NTHREADS, 0, s>>>(v.p, v.x, m.cm[0], m.cm[1], m.xm, c.n);
+  note_launches(1);
   BEM_CUDA_TRY(cudaGetLastError());
   return BEM_OK;
 }
@@ -887,17 +1020,20 @@ void pk_chunk_launches(bem_kernel_s* k, cudaStream_t s) {
   SolveState* st = k->ws.state;
   double* part = k->ws.partials;
   unsigned int* tk = k->ws.ticket;
-  uint8_t* cm = k->ws.mask;   // contact set of the iterations (the adhesive masks are not live here)
+  const PkSets m = pk_sets(k);
+  static_assert(CHUNK % 2 == 0, "a chunk starts and ends on the first set buffer");
   for (int it = 0; it < CHUNK; ++it) {
+    uint8_t *cm = m.cm[it & 1], *other = m.cm[1 - (it & 1)];   // this iteration's set; the previous, then the next one
     launch_matvec<T>(k, v.x, v.u, s, &st->mv_p_on);
-    launch_pdl(k_pk_begin<T>, c.rb, NTHREADS, 0, s, v.p, v.g, (const T*)v.f, v.x, (const T*)v.u, cm, part, tk, st,
-               c.n);
-    launch_pdl(k_pk_dir<T>, c.eb, NTHREADS, 0, s, (const uint8_t*)cm, (const T*)v.g, v.t, (const SolveState*)st, c.n);
+    launch_pdl(k_pk_begin<T>, c.rb, NTHREADS, 0, s, v.p, v.g, (const T*)v.f, v.x, (const T*)v.u, (const uint8_t*)cm,
+               (const uint8_t*)m.xm, part, tk, st, c.n);
+    launch_pdl(k_pk_dir<T>, c.eb, NTHREADS, 0, s, (const uint8_t*)cm, (const uint8_t*)other, (const T*)v.g, v.t,
+               (const SolveState*)st, c.n);
     launch_matvec<T>(k, v.t, v.r, s, &st->mv_t_on);
     launch_pdl(k_pk_rt<T>, sizeof(T) == 4 ? c.rb6 : c.rb, NTHREADS, 0, s, (const uint8_t*)cm, (const T*)v.g,
                (const T*)v.t, (const T*)v.r, part, tk, st, c.n);
     launch_pdl(k_pk_update<T>, c.rb, NTHREADS, 0, s, v.p, v.g, (const T*)v.t, (const T*)v.r, v.x, (const T*)v.f,
-               part, tk, st, c.n);
+               (const uint8_t*)cm, other, m.xm, part, tk, st, c.n);
     note_launches(4);
   }
 }
@@ -1078,9 +1214,9 @@ void lin_chunk_launches(bem_kernel_s* k, const uint8_t* C, cudaStream_t s) {
   unsigned int* tk = k->ws.ticket;
   for (int it = 0; it < CHUNK; ++it) {
     launch_matvec<T>(k, v.t, v.g, s, &st->mv_t_on);
-    launch_pdl(k_lin_alpha<T>, c.rb, NTHREADS, 0, s, (const T*)v.t, (const T*)v.g, (const T*)v.r, C, part, tk, st,
+    launch_pdl(k_lin_alpha<T>, c.rbl, NTHREADS, 0, s, (const T*)v.t, (const T*)v.g, (const T*)v.r, C, part, tk, st,
                c.n);
-    launch_pdl(k_lin_update<T>, c.rb, NTHREADS, 0, s, v.x, v.r, (const T*)v.t, (const T*)v.g, C, part, tk, st, c.n);
+    launch_pdl(k_lin_update<T>, c.rbl, NTHREADS, 0, s, v.x, v.r, (const T*)v.t, (const T*)v.g, C, part, tk, st, c.n);
     launch_pdl(k_lin_dir<T>, c.eb, NTHREADS, 0, s, (const T*)v.r, v.t, C, (const SolveState*)st, c.n);
     note_launches(3);
   }
