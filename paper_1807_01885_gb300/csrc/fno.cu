@@ -1025,6 +1025,8 @@ __global__ void __launch_bounds__(128) k_proj_tc(const float* __restrict__ X, in
 }
 
 // c_k / N^2, the weights of the gradient of the inverse transform, for the current N
+#include "fno_infer.cuh"
+
 __global__ void k_cky_scaled(const float* __restrict__ c, float* __restrict__ cs, int m, float inv) {
   FOR_N(k, (size_t)m) cs[k] = c[k] * inv;
 }
@@ -1382,10 +1384,12 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
   const int nv = train ? L + 1 : 2, nz = train ? L : 1;
   cudaError_t e = cudaSuccess;
   f->v.resize(nv);
-  f->z.resize(nz);
+  f->z.assign(nz, nullptr);
   f->Xh.resize(train ? L : 1);
   for (int i = 0; i < nv && e == cudaSuccess; ++i) e = alloc(f, &f->v[i], (size_t)B * W * P);
-  for (int i = 0; i < nz && e == cudaSuccess; ++i) e = alloc(f, &f->z[i], (size_t)B * W * P);
+  // (the fused layers keep z only for the backward pass)
+  const bool keep_z = train || !fused_ok(f) || (size_t)W * P >= (size_t(1) << 32);
+  for (int i = 0; i < nz && e == cudaSuccess && keep_z; ++i) e = alloc(f, &f->z[i], (size_t)B * W * P);
   for (size_t i = 0; i < f->Xh.size() && e == cudaSuccess; ++i) e = alloc(f, &f->Xh[i], (size_t)B * W * nm);
   const bool hidden = !proj_ok(f, N);   // the hidden layer is stored
   if (e == cudaSuccess && hidden) e = alloc(f, &f->a, (size_t)B * H * P);
@@ -1710,6 +1714,51 @@ bem_status forward(bem_fno_s* f, int B, int N, const float* x, bool train, cudaS
   return BEM_OK;
 }
 
+// the one-pass inference (fno_infer.cuh): whole 16-pixel tiles, at most 16 modes
+bool infer_ok(const bem_fno_s* f, int N) {
+  return fused_size(f, N) && proj_ok(f, N) && N % 16 == 0 && N <= kInfMaxN && f->d.modes <= 16;
+}
+
+template <int KT, int NT, int KS>
+void infer_run(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
+  const int W = f->d.width, L = f->d.layers, n2m = 2 * f->d.modes;
+  const size_t rows = (size_t)B * N, warps = rows * infer_chunks(N / 16);
+  const unsigned grid = (unsigned)((warps + 3) / 4);
+  float* A = reinterpret_cast<float*>(f->A);
+  uint2* v[2] = {reinterpret_cast<uint2*>(f->v[0]), reinterpret_cast<uint2*>(f->v[1])};
+  const bf16* wb = f->wb;
+  k_lift_inf<NT, 2 * KS><<<grid, 128, 0, s>>>(x, wb + f->o_Pw, wb + f->o_Pb, f->TfB, v[0], A, N, n2m, rows);
+  note_launches(1);
+  for (int l = 0; l < L; ++l) {
+    modes_x<false>(f, l, f->Xh[0], nullptr, B, N, s);
+    const bf16 *Ww = wb + f->o_Ww + (size_t)l * W * W, *Wb = wb + f->o_Wb + (size_t)l * W;
+    const uint2* vin = v[l & 1];
+    if (l < L - 1)
+      k_layer_inf<KT, NT, KS, false><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, v[1 - (l & 1)],
+                                                          nullptr, nullptr, nullptr, nullptr, 0, nullptr, N, n2m, rows);
+    else
+      k_layer_inf<KT, NT, KS, true><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, nullptr,
+                                                         wb + f->o_Q1w, wb + f->o_Q1b, wb + f->o_Q2w, wb + f->o_Q2b,
+                                                         f->d.hidden, out, N, n2m, rows);
+    note_launches(1);
+  }
+}
+
+template <int KT, int NT>
+void infer_ks(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
+  if (f->d.modes <= 8) infer_run<KT, NT, 1>(f, B, N, x, out, s);
+  else infer_run<KT, NT, 2>(f, B, N, x, out, s);
+}
+
+// out = network(x) (infer_ok)
+bem_status infer(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
+  if (f->d.width == 8) infer_ks<1, 1>(f, B, N, x, out, s);
+  else if (f->d.width == 16) infer_ks<1, 2>(f, B, N, x, out, s);
+  else infer_ks<2, 4>(f, B, N, x, out, s);
+  BEM_CUDA_TRY(cudaGetLastError());
+  return BEM_OK;
+}
+
 bem_status backward(bem_fno_s* f, int B, int N, const float* x, const float* target, double* loss, cudaStream_t s) {
   const int W = f->d.width, m = f->d.modes, L = f->d.layers, H = f->d.hidden;
   const size_t P = (size_t)N * N, nm = 2 * (size_t)m * m, bc = (size_t)B * W;
@@ -1923,6 +1972,7 @@ bem_status bem_fno_forward(bem_fno f, int32_t B, int32_t N, const float* x, floa
   cudaStream_t s = (cudaStream_t)cuda_stream;
   bem_status st = ensure(f, B, N, f->cap_train && B <= f->capB && N <= f->capN, s);
   if (st != BEM_OK) return st;
+  if (infer_ok(f, N)) return infer(f, B, N, x, out, s);
   st = forward(f, B, N, x, f->cap_train, s);
   if (st != BEM_OK) return st;
   BEM_CUDA_TRY(cudaMemcpyAsync(out, f->out, (size_t)B * N * N * sizeof(float), cudaMemcpyDeviceToDevice, s));
