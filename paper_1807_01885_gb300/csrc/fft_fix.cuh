@@ -321,12 +321,21 @@ __device__ __forceinline__ DD dd_mul(DD a, DD b) {
   const double h = p + e;
   return DD{h, e - (h - p)};
 }
-__device__ __forceinline__ DD dd_div(DD a, double b) {
-  const double q = a.h / b;
-  const double r = fma(-q, b, a.h) + a.l;
-  const double q2 = r / b, h = q + q2;
-  return DD{h, q2 - (h - q)};
-}
+// (-1)^k / (2k)! and (-1)^k / (2k + 1)!: the Taylor coefficients of cos and of sin(x)/x in x^2
+static __constant__ double c_cos[12][2] = {
+    {1.0, 0.0}, {-0.5, 0.0}, {0.041666666666666664, 2.3129646346357427e-18}, {-0.001388888888888889,
+    5.300543954373577e-20}, {2.48015873015873e-05, 2.1511947866775882e-23}, {-2.755731922398589e-07,
+    -2.3767714622250297e-23}, {2.08767569878681e-09, -1.20734505911326e-25}, {-1.1470745597729725e-11,
+    -2.0655512752830745e-28}, {4.779477332387385e-14, 4.399205485834081e-31}, {-1.5619206968586225e-16,
+    -1.1910679660273754e-32}, {4.110317623312165e-19, 1.4412973378659527e-36}, {-8.896791392450574e-22,
+    7.911402614872376e-38}};
+static __constant__ double c_sin[12][2] = {
+    {1.0, 0.0}, {-0.16666666666666666, -9.25185853854297e-18}, {0.008333333333333333, 1.1564823173178714e-19},
+    {-0.0001984126984126984, -1.7209558293420705e-22}, {2.7557319223985893e-06, -1.858393274046472e-22},
+    {-2.505210838544172e-08, 1.448814070935912e-24}, {1.6059043836821613e-10, 1.2585294588752098e-26},
+    {-7.647163731819816e-13, -7.03872877733453e-30}, {2.8114572543455206e-15, 1.6508842730861433e-31},
+    {-8.22063524662433e-18, -2.2141894119604265e-34}, {1.9572941063391263e-20, -1.3643503830087908e-36},
+    {-3.868170170630684e-23, 8.843177655482344e-40}};
 __device__ __forceinline__ i64 dd_fix(DD v) {   // v 2^62, rounded
   const double s = 4611686018427387904.0;
   const i64 a = __double2ll_rn(v.h * s);
@@ -340,13 +349,13 @@ __device__ inline int4 fix_twiddle(int num, int den) {
   if (oct & 1) rn = den - rn;
   const DD pi4 = DD{0.78539816339744830962, 3.0616169978683829431e-17};
   const DD x = dd_mul(DD{(double)rn / (double)den, 0.0}, pi4), x2 = dd_mul(x, x);
-  DD c = DD{1.0, 0.0}, s = x, tc = DD{1.0, 0.0}, ts = x;
-  for (int k = 1; k <= 11; ++k) {
-    tc = dd_div(dd_mul(tc, x2), -(double)((2 * k - 1) * (2 * k)));
-    ts = dd_div(dd_mul(ts, x2), -(double)((2 * k) * (2 * k + 1)));
-    c = dd_add(c, tc);
-    s = dd_add(s, ts);
+  DD c = DD{c_cos[11][0], c_cos[11][1]}, s = DD{c_sin[11][0], c_sin[11][1]};
+#pragma unroll 1
+  for (int k = 10; k >= 0; --k) {
+    c = dd_add(dd_mul(c, x2), DD{c_cos[k][0], c_cos[k][1]});
+    s = dd_add(dd_mul(s, x2), DD{c_sin[k][0], c_sin[k][1]});
   }
+  s = dd_mul(s, x);
   i64 C = dd_fix(c), S = dd_fix(s);
   const int q = (oct + 1) >> 1;                     // quarter turns added to +-r
   if (oct & 1) S = -S;

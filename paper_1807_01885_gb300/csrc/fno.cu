@@ -1198,6 +1198,44 @@ __global__ void __launch_bounds__(256) k_dft_x_any(const float2* __restrict__ A,
 
 #include "fno_modes.cuh"
 
+// Y[b][o][mode] = sum_i X[b][i][mode] R[i][o][mode]
+__global__ void k_mix(const float2* __restrict__ X, const bf16* __restrict__ Rre, const bf16* __restrict__ Rim,
+                      float2* __restrict__ Y, int W, int nm, int B) {
+  FOR_N(e, (size_t)B * W * nm) {
+    const int mode = (int)(e % nm);
+    const int o = (int)((e / nm) % W);
+    const int b = (int)(e / ((size_t)nm * W));
+    float re = 0.f, im = 0.f;
+    for (int i = 0; i < W; ++i) {
+      const float2 x = X[((size_t)b * W + i) * nm + mode];
+      const size_t r = ((size_t)i * W + o) * nm + mode;
+      const float rr = b2f(Rre[r]), ri = b2f(Rim[r]);
+      re += x.x * rr - x.y * ri;
+      im += x.x * ri + x.y * rr;
+    }
+    Y[e] = make_float2(re, im);
+  }
+}
+
+// dX[b][i][mode] = sum_o conj(R[i][o][mode]) dY[b][o][mode]
+__global__ void k_mix_dgrad(const float2* __restrict__ dY, const bf16* __restrict__ Rre, const bf16* __restrict__ Rim,
+                            float2* __restrict__ dX, int W, int nm, int B) {
+  FOR_N(e, (size_t)B * W * nm) {
+    const int mode = (int)(e % nm);
+    const int i = (int)((e / nm) % W);
+    const int b = (int)(e / ((size_t)nm * W));
+    float re = 0.f, im = 0.f;
+    for (int o = 0; o < W; ++o) {
+      const float2 d = dY[((size_t)b * W + o) * nm + mode];
+      const size_t r = ((size_t)i * W + o) * nm + mode;
+      const float rr = b2f(Rre[r]), ri = b2f(Rim[r]);
+      re += rr * d.x + ri * d.y;
+      im += rr * d.y - ri * d.x;
+    }
+    dX[e] = make_float2(re, im);
+  }
+}
+
 // dR[i][o][mode] = sum_b conj(X[b][i][mode]) dY[b][o][mode]
 __global__ void k_mix_wgrad(const float2* __restrict__ X, const float2* __restrict__ dY, float* __restrict__ gre,
                             float* __restrict__ gim, int W, int nm, int B) {
@@ -1306,7 +1344,7 @@ struct bem_fno_s {
   float *a = nullptr, *h = nullptr, *out = nullptr, *dout = nullptr;
   float *dv = nullptr, *dz = nullptr, *dt = nullptr, *mom = nullptr, *part = nullptr, *part2 = nullptr, *cky = nullptr, *cky_s = nullptr;
   double* mom_part = nullptr;   // per-chunk sums of the height moments
-  float2 *A = nullptr, *Y = nullptr, *dY = nullptr, *Xp = nullptr, *tw = nullptr, *twx = nullptr;
+  float2 *A = nullptr, *Y = nullptr, *dY = nullptr, *tw = nullptr, *twx = nullptr;
   float *Tf = nullptr, *Ti = nullptr;   // twiddle matrices of the y transforms (N x 2m, 2m x N)
   uint4 *TfB = nullptr, *TiB = nullptr; // the same split into bf16 hi/lo, in mma fragment order
   uint4* TfA = nullptr;                 // Tf split, in A-fragment order (fused layer kernel)
@@ -1403,7 +1441,6 @@ bem_status ensure(bem_fno_s* f, int B, int N, bool train, cudaStream_t s) {
   if (e == cudaSuccess) e = alloc(f, &f->A, (size_t)B * W * N * m);
   if (e == cudaSuccess) e = alloc(f, &f->Y, (size_t)B * W * nm);
   if (e == cudaSuccess) e = alloc(f, &f->dY, (size_t)B * W * nm);
-  if (e == cudaSuccess) e = alloc(f, &f->Xp, (kXBlocks + (size_t)B * W) * nm);   // dft_x_chunks(bc) bc <= kXBlocks + bc
   if (e == cudaSuccess) e = alloc(f, &f->tw, (size_t)N);
   if (e == cudaSuccess) e = alloc(f, &f->twx, (size_t)N * dft_x_kt(m));
   if (e == cudaSuccess) e = alloc(f, &f->Tf, (size_t)2 * m * N);
@@ -1542,16 +1579,17 @@ void modes_x(bem_fno_s* f, int l, float2* Xh, const float* wky, int B, int N, cu
   const size_t bc = (size_t)B * W, nm = 2 * (size_t)m * m;
   const bf16* Rre = f->wb + f->o_Rre + (size_t)l * W * W * nm;
   const bf16* Rim = f->wb + f->o_Rim + (size_t)l * W * W * nm;
-  const bool tiled = m <= kXModes;
-  const int chunks = tiled ? dft_x_chunks(bc, N, m) : 1;
-  float2* Xp = chunks > 1 ? f->Xp : Xh;
-  if (tiled) k_dft_x<<<dim3((unsigned)bc, chunks), 256, 0, s>>>(f->A, Xp, f->twx, wky, N, m);
-  else k_dft_x_any<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, Xp, f->tw, wky, N, m);
-  mix<CONJ>(Xp, chunks, Xh, Rre, Rim, f->Y, W, (int)nm, B, s);
-  if (tiled)
+  if (dft_x_tiled(bc, m)) {
+    const DftX d(m);
+    k_dft_x<<<(unsigned)bc, ((d.SB * d.items + 31) / 32) * 32, 0, s>>>(f->A, Xh, f->twx, wky, N, m);
+  } else {
+    k_dft_x_any<<<dim3((unsigned)bc, 2 * m), 256, 0, s>>>(f->A, Xh, f->tw, wky, N, m);
+  }
+  if (CONJ) k_mix_dgrad<<<blocks_for(bc * nm), FT, 0, s>>>(Xh, Rre, Rim, f->Y, W, (int)nm, B);
+  else k_mix<<<blocks_for(bc * nm), FT, 0, s>>>(Xh, Rre, Rim, f->Y, W, (int)nm, B);
+  if (idft_x_tiled(bc, m, N))
     k_idft_x<<<dim3((unsigned)bc, (N + kXRows - 1) / kXRows), ((m + 1) / 2) * (kXRows / 4) > 128 ? 256 : 128,
-             idft_x_smem(m), s>>>(
-        f->Y, f->A, f->twx, N, m);
+             idft_x_smem(m), s>>>(f->Y, f->A, f->twx, N, m);
   else
     k_idft_x_any<<<blocks_for(bc * N * ((m + 3) / 4)), FT, 0, s>>>(f->Y, f->A, f->tw, N, m, bc);
   note_launches(3);
@@ -1719,35 +1757,44 @@ bool infer_ok(const bem_fno_s* f, int N) {
   return fused_size(f, N) && proj_ok(f, N) && N % 16 == 0 && N <= kInfMaxN && f->d.modes <= 16;
 }
 
-template <int KT, int NT, int KS>
+template <int KT, int NT, int KS, int CH>
 void infer_run(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
   const int W = f->d.width, L = f->d.layers, n2m = 2 * f->d.modes;
-  const size_t rows = (size_t)B * N, warps = rows * infer_chunks(N / 16);
+  const size_t rows = (size_t)B * N, warps = rows * CH;
   const unsigned grid = (unsigned)((warps + 3) / 4);
   float* A = reinterpret_cast<float*>(f->A);
   uint2* v[2] = {reinterpret_cast<uint2*>(f->v[0]), reinterpret_cast<uint2*>(f->v[1])};
   const bf16* wb = f->wb;
-  k_lift_inf<NT, 2 * KS><<<grid, 128, 0, s>>>(x, wb + f->o_Pw, wb + f->o_Pb, f->TfB, v[0], A, N, n2m, rows);
+  k_lift_inf<NT, 2 * KS, CH><<<grid, 128, 0, s>>>(x, wb + f->o_Pw, wb + f->o_Pb, f->TfB, v[0], A, N, n2m, rows);
   note_launches(1);
   for (int l = 0; l < L; ++l) {
     modes_x<false>(f, l, f->Xh[0], nullptr, B, N, s);
     const bf16 *Ww = wb + f->o_Ww + (size_t)l * W * W, *Wb = wb + f->o_Wb + (size_t)l * W;
     const uint2* vin = v[l & 1];
     if (l < L - 1)
-      k_layer_inf<KT, NT, KS, false><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, v[1 - (l & 1)],
-                                                          nullptr, nullptr, nullptr, nullptr, 0, nullptr, N, n2m, rows);
+      k_layer_inf<KT, NT, KS, false, CH><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, v[1 - (l & 1)],
+                                                              nullptr, nullptr, nullptr, nullptr, 0, nullptr, N, n2m,
+                                                              rows);
     else
-      k_layer_inf<KT, NT, KS, true><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, nullptr,
-                                                         wb + f->o_Q1w, wb + f->o_Q1b, wb + f->o_Q2w, wb + f->o_Q2b,
-                                                         f->d.hidden, out, N, n2m, rows);
+      k_layer_inf<KT, NT, KS, true, CH><<<grid, 128, 0, s>>>(vin, Ww, Wb, A, f->cky_s, f->TfA, f->TfB, nullptr,
+                                                             wb + f->o_Q1w, wb + f->o_Q1b, wb + f->o_Q2w,
+                                                             wb + f->o_Q2b, f->d.hidden, out, N, n2m, rows);
     note_launches(1);
   }
 }
 
+template <int KT, int NT, int KS>
+void infer_ch(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
+  switch (infer_chunks(N / 16)) {
+    case 1: infer_run<KT, NT, KS, 1>(f, B, N, x, out, s); break;
+    case 2: infer_run<KT, NT, KS, 2>(f, B, N, x, out, s); break;
+    default: infer_run<KT, NT, KS, 4>(f, B, N, x, out, s); break;
+  }
+}
 template <int KT, int NT>
 void infer_ks(bem_fno_s* f, int B, int N, const float* x, float* out, cudaStream_t s) {
-  if (f->d.modes <= 8) infer_run<KT, NT, 1>(f, B, N, x, out, s);
-  else infer_run<KT, NT, 2>(f, B, N, x, out, s);
+  if (f->d.modes <= 8) infer_ch<KT, NT, 1>(f, B, N, x, out, s);
+  else infer_ch<KT, NT, 2>(f, B, N, x, out, s);
 }
 
 // out = network(x) (infer_ok)

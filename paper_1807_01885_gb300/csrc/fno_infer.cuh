@@ -10,24 +10,29 @@
 // rows it produces (the next layer's spectral input) from the parts it just made, and the
 // last layer goes straight through the projection, so per layer the activations are read
 // once and written once and the last ones never leave the SM.
-// Measured on GB300 (32 channels, 16 modes, 4 layers, one sample of N = 2048): @INF@.
+// Measured on GB300 (32 channels, 16 modes, 4 layers, one sample of N = 2048): forward 3.02
+// -> 1.85 ms; a layer 345 us (1.07 GB) where layer and transform took 520; three blocks of
+// 168 registers per SM against four of 128 1.81 / 1.93 ms, two 1.88.
 #pragma once
 
 constexpr int kInfRow = 20;          // records per staged row of 16 pixels (160 bytes: conflict-free operand reads)
 constexpr int kInfMaxN = 2048;       // at most four chunks of 32 tiles per row, one per warp of a block
 
 // chunks of a row of YT tiles: 1, 2 or 4, so that a block's four warps hold whole rows
-__host__ __device__ inline int infer_chunks(int YT) { return YT <= 32 ? 1 : (YT <= 64 ? 2 : 4); }
+inline int infer_chunks(int YT) { return YT <= 32 ? 1 : (YT <= 64 ? 2 : 4); }
 
-// transforms along y of a tile's 16 pixels x W channels, added to acc: hp / lp [nt][h] are
-// the packed channel pairs 8 nt + 2t, + 1 of pixel g + 8 h
-template <int NT, int NM>
-__device__ __forceinline__ void tile_dft(float (&acc)[(NT + 1) / 2][NM][4], const unsigned (&hp)[NT][2],
-                                         const unsigned (&lp)[NT][2], const uint4* __restrict__ TfB, int yt, int nm,
-                                         int lane) {
-  uint4 b[NM];
+// the transform's operand fragments of tile yt (nm column blocks of them)
+template <int NM>
+__device__ __forceinline__ void load_dft(uint4 (&b)[NM], const uint4* __restrict__ TfB, int yt, int nm, int lane) {
 #pragma unroll
   for (int j = 0; j < NM; ++j) b[j] = j < nm ? __ldg(TfB + ((size_t)yt * nm + j) * 32 + lane) : make_uint4(0, 0, 0, 0);
+}
+
+// transforms along y of a tile's 16 pixels x W channels, added to acc: hp / lp [nt][h] are
+// the packed channel pairs 8 nt + 2t, + 1 of pixel g + 8 h; b from load_dft
+template <int NT, int NM>
+__device__ __forceinline__ void tile_dft(float (&acc)[(NT + 1) / 2][NM][4], const unsigned (&hp)[NT][2],
+                                         const unsigned (&lp)[NT][2], const uint4 (&b)[NM], int nm) {
 #pragma unroll
   for (int mt = 0; mt < (NT + 1) / 2; ++mt) {
     // rows = channels 16 mt + g (+ 8), k = pixels: the 8 x 8 blocks transposed
@@ -52,9 +57,9 @@ __device__ __forceinline__ void tile_dft(float (&acc)[(NT + 1) / 2][NM][4], cons
 
 // adds the chunks' transforms of the block's rows (in chunk order) and writes them:
 // A[((b W + o) N + x) n2m + k]; red: 4 x 16 MT x 8 NM floats
-template <int NT, int NM>
+template <int NT, int NM, int CH>
 __device__ __forceinline__ void store_dft(const float (&acc)[(NT + 1) / 2][NM][4], float* red, float* __restrict__ A,
-                                          int chunks, size_t row, size_t rows, int N, int n2m, int lane, int wid) {
+                                          size_t row, size_t rows, int N, int n2m, int lane, int wid) {
   constexpr int W = 8 * NT, K = 8 * NM;
   const int g = lane / 4, t = lane % 4;
   __syncthreads();   // the staging buffers that red overlays have been read
@@ -70,22 +75,22 @@ __device__ __forceinline__ void store_dft(const float (&acc)[(NT + 1) / 2][NM][4
       }
   __syncthreads();
   if (row >= rows) return;
-  const int chunk = wid % chunks;
+  const int chunk = wid % CH;
   const size_t b = row / N;
   const int x = (int)(row % N);
   const float* first = red + (wid - chunk) * W * K;
   // the row's warps share the outputs
-  for (int i = chunk * 32 + lane; i < W * K; i += chunks * 32) {
+  for (int i = chunk * 32 + lane; i < W * K; i += CH * 32) {
     const int o = i / K, k = i % K;
     if (k >= n2m) continue;
     float s = first[i];
-    for (int c = 1; c < chunks; ++c) s += first[c * W * K + i];
+    for (int c = 1; c < CH; ++c) s += first[c * W * K + i];
     A[((b * W + o) * N + x) * n2m + k] = s;
   }
 }
 
 // v0 = P x + p in records, and its transform along y
-template <int NT, int NM>
+template <int NT, int NM, int CH>
 __global__ void __launch_bounds__(128, 4) k_lift_inf(const float* __restrict__ X, const bf16* __restrict__ Pw,
                                                      const bf16* __restrict__ Pb, const uint4* __restrict__ TfB,
                                                      uint2* __restrict__ V, float* __restrict__ A, int N, int n2m,
@@ -93,9 +98,9 @@ __global__ void __launch_bounds__(128, 4) k_lift_inf(const float* __restrict__ X
   constexpr int W = 8 * NT, MT = (NT + 1) / 2;
   __shared__ float red[4 * W * 8 * NM];
   const int lane = threadIdx.x % 32, g = lane / 4, t = lane % 4, wid = threadIdx.x / 32;
-  const int YT = N / 16, chunks = infer_chunks(YT), tpw = (YT + chunks - 1) / chunks;
-  const size_t row = ((size_t)blockIdx.x * 4 + wid) / chunks;
-  const int chunk = wid % chunks;
+  const int YT = N / 16, tpw = (YT + CH - 1) / CH;
+  const size_t row = ((size_t)blockIdx.x * 4 + wid) / CH;
+  const int chunk = wid % CH;
   float dacc[MT][NM][4] = {};
   if (row < rows) {
     const size_t b = row / N, P = (size_t)N * N, base = (row % N) * (size_t)N;
@@ -123,6 +128,8 @@ __global__ void __launch_bounds__(128, 4) k_lift_inf(const float* __restrict__ X
     if (yt0 < yt1) load(yt0, cur);
     for (int yt = yt0; yt < yt1; ++yt) {
       if (yt + 1 < yt1) load(yt + 1, nxt);
+      uint4 tb[NM];
+      load_dft<NM>(tb, TfB, yt, (n2m + 7) / 8, lane);
       unsigned ah[4] = {0u, 0u, 0u, 0u}, al[4] = {0u, 0u, 0u, 0u};
       split2(cur[0], cur[1], ah[0], al[0]);
       split2(cur[2], cur[3], ah[1], al[1]);
@@ -138,19 +145,19 @@ __global__ void __launch_bounds__(128, 4) k_lift_inf(const float* __restrict__ X
           vp[(size_t)(4 * nt) * P + 16 * yt + 8 * h] = make_uint2(hp[nt][h], lp[nt][h]);
         }
       }
-      tile_dft<NT, NM>(dacc, hp, lp, TfB, yt, (n2m + 7) / 8, lane);
+      tile_dft<NT, NM>(dacc, hp, lp, tb, (n2m + 7) / 8);
 #pragma unroll
       for (int e = 0; e < 4; ++e) cur[e] = nxt[e];
     }
   }
-  store_dft<NT, NM>(dacc, red, A, chunks, row, rows, N, n2m, lane, wid);
+  store_dft<NT, NM, CH>(dacc, red, A, row, rows, N, n2m, lane, wid);
 }
 
 // One Fourier layer on records (the arithmetic of k_layer_tc).  LAST false: v' = gelu(z)
 // in records and its transform along y; LAST true: z through the projection (the
 // arithmetic of k_proj_tc) into out.
-template <int KT, int NT, int KS, bool LAST>
-__global__ void __launch_bounds__(128, 4)
+template <int KT, int NT, int KS, bool LAST, int CH>
+__global__ void __launch_bounds__(128, 3)
 k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16* __restrict__ Wb, float* A,
             const float* __restrict__ cs, const uint4* __restrict__ TfA, const uint4* __restrict__ TfB,
             uint2* __restrict__ Vout, const bf16* __restrict__ Q1, const bf16* __restrict__ q1,
@@ -164,9 +171,9 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
   __shared__ float2 sqb[LAST ? 8 * 4 : 1], sqw[LAST ? 8 * 4 : 1];
   uint2(*stage)[2][STAGE] = reinterpret_cast<uint2(*)[2][STAGE]>(raw);
   const int lane = threadIdx.x % 32, g = lane / 4, t = lane % 4, wid = threadIdx.x / 32;
-  const int YT = N / 16, chunks = infer_chunks(YT), tpw = (YT + chunks - 1) / chunks;
-  const size_t row = ((size_t)blockIdx.x * 4 + wid) / chunks;
-  const int chunk = wid % chunks;
+  const int YT = N / 16, tpw = (YT + CH - 1) / CH;
+  const size_t row = ((size_t)blockIdx.x * 4 + wid) / CH;
+  const int chunk = wid % CH;
   const int nh = (H + 7) / 8;
   if constexpr (LAST) {
     for (int i = threadIdx.x; i < KT * nh * 32; i += 128) {
@@ -237,9 +244,26 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
       cp_async_commit();
     };
     const int yt0 = chunk * tpw, yt1 = min(YT, yt0 + tpw);
-    if (yt0 < yt1) prefetch(yt0, 0);
+    // the inverse transform's pixel operand, loaded a tile ahead (the unit's waits for these
+    // loads were the kernel's largest stall)
+    unsigned th[KS][4], tl[KS][4];
+    auto load_inv = [&](int yt) {
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        const uint4* tp = TfA + (((size_t)yt * KS + ks) * 32 + lane) * 2;
+        const uint4 h4 = __ldg(tp), l4 = __ldg(tp + 1);
+        th[ks][0] = h4.x; th[ks][1] = h4.y; th[ks][2] = h4.z; th[ks][3] = h4.w;
+        tl[ks][0] = l4.x; tl[ks][1] = l4.y; tl[ks][2] = l4.z; tl[ks][3] = l4.w;
+      }
+    };
+    if (yt0 < yt1) {
+      prefetch(yt0, 0);
+      load_inv(yt0);
+    }
     for (int yt = yt0; yt < yt1; ++yt) {
       const int i = yt - yt0;
+      [[maybe_unused]] uint4 tb[LAST ? 1 : NM];
+      if constexpr (!LAST) load_dft<NM>(tb, TfB, yt, (n2m + 7) / 8, lane);
       if (yt + 1 < yt1) prefetch(yt + 1, (i + 1) & 1);
       else cp_async_commit();
       cp_async_wait<1>();
@@ -257,14 +281,6 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
           al[kb][e] = r.y;
         }
       __syncwarp();   // every lane has read the stage before it is refilled
-      unsigned th[KS][4], tl[KS][4];
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        const uint4* tp = TfA + (((size_t)yt * KS + ks) * 32 + lane) * 2;
-        const uint4 h4 = __ldg(tp), l4 = __ldg(tp + 1);
-        th[ks][0] = h4.x; th[ks][1] = h4.y; th[ks][2] = h4.z; th[ks][3] = h4.w;
-        tl[ks][0] = l4.x; tl[ks][1] = l4.y; tl[ks][2] = l4.z; tl[ks][3] = l4.w;
-      }
       unsigned hp[NT][2], lp[NT][2];
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
@@ -294,8 +310,9 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
             vo[(size_t)(4 * nt) * P + 16 * yt + 8 * h] = make_uint2(hp[nt][h], lp[nt][h]);
         }
       }
+      if (yt + 1 < yt1) load_inv(yt + 1);
       if constexpr (!LAST) {
-        tile_dft<NT, NM>(dacc, hp, lp, TfB, yt, (n2m + 7) / 8, lane);
+        tile_dft<NT, NM>(dacc, hp, lp, tb, (n2m + 7) / 8);
       } else {
         float sa = 0.f, sb2 = 0.f;
         for (int j = 0; j < nh; ++j) {
@@ -333,5 +350,5 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
     cp_async_wait<0>();
   }
   if constexpr (!LAST)
-    store_dft<NT, NM>(dacc, reinterpret_cast<float*>(raw), A, chunks, row, rows, N, n2m, lane, wid);
+    store_dft<NT, NM, CH>(dacc, reinterpret_cast<float*>(raw), A, row, rows, N, n2m, lane, wid);
 }
