@@ -198,7 +198,8 @@ def fp64_bench(torch, bem, inst, stream, reps=20):
     tf = fft_nominal_flops(N) / (ms * 1e-3) / 1e12
     return {"ms_per_matvec": ms, "nominal_gflop": fft_nominal_flops(N) / 1e9, "tflops": tf,
             "dgemm_tflops_measured": gemm, "frac_of_dgemm": tf / gemm,
-            "note": "FP64 product (nominal transform flops) against cuBLAS DGEMM 4096^3 in the same run"}
+            "note": "double product (nominal transform flops) against cuBLAS DGEMM 4096^3 in the same run; the "
+                    "product runs on 64-bit fixed-point transforms, not on the FP64 pipe, so the fraction may pass 1"}
 
 
 class Clocks:

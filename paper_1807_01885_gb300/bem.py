@@ -170,15 +170,22 @@ def _ptr(x):
     raise TypeError(f"unsupported array type {type(x)}")
 
 
+_current_stream = None
+
+
 def _stream(stream):
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
-        return None
+        # torch and its answer on whether there is a GPU are looked up once: they cost a
+        # call more than its launch does
+        global _current_stream
+        if _current_stream is None:
+            try:
+                import torch
+                if torch.cuda.is_available():
+                    _current_stream = torch.cuda.current_stream
+            except ImportError:
+                pass
+        return None if _current_stream is None else _current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

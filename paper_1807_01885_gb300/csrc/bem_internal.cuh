@@ -285,6 +285,9 @@ template <typename T>
 void reg_twiddles(const bem_kernel_s* k, cudaStream_t s);
 template <typename T>
 void reg_prepare(const bem_kernel_s* k);
+// matvec_f32.cu: bem_matvec's product in one launch where the grid is small
+bool small_product_ok(const bem_kernel_s* k);
+void small_product(const bem_kernel_s* k, const float* p, float* u, cudaStream_t s);
 // matvec_fix.cu (double, N >= 16): one pass of the fixed-point product, its twiddles
 void fix_pass(const bem_kernel_s* k, int which, const double* p, double* u, cudaStream_t s);
 void fix_twiddles(const bem_kernel_s* k, cudaStream_t s);

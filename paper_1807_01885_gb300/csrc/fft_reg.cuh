@@ -294,11 +294,12 @@ __device__ __forceinline__ void apply_twiddles(const C* tws, int ns, int k, X&& 
 
 // Synchronisation of the threads of one transform around its exchanges.  When a
 // block holds several transforms, each exchanges through its own buffer, so it
-// waits only for its own threads: one warp (__syncwarp), or a named barrier per
+// waits only for its own threads: those of one warp (__syncwarp), or a named barrier per
 // transform (ids 1..15, id 0 being __syncthreads); otherwise the whole block.
 template <int TT, int PER_BLOCK>
 struct GroupSync {
-  static constexpr int kind = (PER_BLOCK == 1) ? 0 : (TT == 32 ? 1 : ((TT > 32 && PER_BLOCK <= 15) ? 2 : 0));
+  static constexpr int kind =
+      (PER_BLOCK == 1) ? 0 : (TT <= 32 && TT * PER_BLOCK % 32 == 0 ? 1 : ((TT > 32 && PER_BLOCK <= 15) ? 2 : 0));
   __device__ __forceinline__ static void sync(int group) {
     if constexpr (kind == 1) {
       __syncwarp();

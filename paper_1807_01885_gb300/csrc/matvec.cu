@@ -557,6 +557,14 @@ void launch_pass(const bem_kernel_s* k, int pass, const T* p, T* u, cudaStream_t
 
 template <typename T>
 void launch_product(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4) {
+    // one launch on a small grid (the passes keep their own where they are timed)
+    if (!k->timing.on && small_product_ok(k)) {
+      small_product(k, p, u, s);
+      note_launches(1);
+      return;
+    }
+  }
   run_passes(k, s, [&](int pass) { launch_pass<T>(k, pass, p, u, s); });
 }
 

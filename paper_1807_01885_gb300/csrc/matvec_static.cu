@@ -155,7 +155,7 @@ extern "C" bem_status bem_matvec_static(const bem_kernel_desc* desc, const float
   cudaStream_t s = (cudaStream_t)cuda_stream;
   st = build_table(&k, s);
   if (st != BEM_OK) return st;
-  launch_matvec<float>(&k, p, u, s, nullptr);
+  launch_product<float>(&k, p, u, s);
   BEM_CUDA_TRY(cudaGetLastError());
   return BEM_OK;
 }
