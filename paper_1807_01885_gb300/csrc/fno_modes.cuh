@@ -13,9 +13,10 @@
 // inverse one the kept wave numbers in the order of their index.  (Sharing the products
 // with cos and sin between the sums of +k and -k needs 40 % of the multiply-adds, but
 // rounds differently, and a network's output can be a small difference of its hidden
-// values: a pressure cut at zero then moved by up to 1e-4 of its rms.)
-// Measured on GB300, 1024 channels of N = 256, m = 16, one thread per output with a twiddle
-// load per product / tiled: forward 160 / 75 us, inverse 120 / 38 us.
+// values: a pressure cut at zero then moved by up to 1e-3 of its rms.)
+// Measured on GB300, 512 channels of N = 256, m = 16, one thread per output with a twiddle
+// load per product / tiled: forward 80 / 43 us, inverse 60 / 22 us (1024 channels, tiled:
+// 75 and 38).
 #pragma once
 
 constexpr int kXRows = 64;        // rows x per block of the inverse
@@ -51,7 +52,7 @@ struct DftX {
   __host__ __device__ int groups() const { return (S + SB - 1) / SB; }
 };
 // Where the tiled kernels are the faster ones.  Forward: a block per channel has to fill the
-// GPU and the modes its threads (m = 16, N = 256, 512 channels: 80 -> 38 us; predictions of
+// GPU and the modes its threads (m = 16, N = 256, 512 channels: 80 -> 43 us; predictions of
 // one sample of N = 164, m = 8, were 30 % slower with it, 32 channels of N = 2048 5 %).
 // Inverse: the same for blocks of 64 rows.
 inline bool dft_x_tiled(size_t bc, int m) { return m >= 12 && m <= kXModes && bc >= 304; }

@@ -113,8 +113,8 @@ __device__ __forceinline__ void finish(SolveState* st, int status) {
 // a contact cell then cost their byte word (and, where the gap itself moves, the gap's
 // arrays): 340 -> 150 MB per iteration at N = 2048, and in double the arithmetic of the
 // sums, which bounds those sweeps.  The sums only lose zeros: results are unchanged.
-// Measured on GB300, full sweeps / this: rough surface N = 2048 float 21.6 / 20.4 ms, sphere
-// N = 64 double 5.0 / 4.5, batch of 32 uneven grids 30.7 / 28.6.
+// Measured on GB300, full sweeps / this: sphere N = 64 double 5.04 / 4.53 ms, rough surface
+// N = 2048 float 21.6 / 20.5 ms; a batch of 32 uneven grids gained 3 to 9 %.
 template <typename T>
 __device__ __forceinline__ void stm4(uint8_t* m, size_t i4, const T (&pv)[4]) {
   reinterpret_cast<uchar4*>(m)[i4] =
