@@ -33,6 +33,12 @@ struct Small {
   static constexpr size_t SMEM = (size_t)PC * N * sizeof(float4) + (EX_R > EX_C ? EX_R : EX_C);
 };
 
+// A block's shared memory may be written by its peers only once it has started: every
+// thread of the cluster arrives on entry, and waits before the first remote store.  The
+// arrival publishes nothing (relaxed); the wait hides behind the row transform.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+
 template <int LOGN>
 __global__ void __cluster_dims__(Small<LOGN>::CTAS, 1, 1) __launch_bounds__(Small<LOGN>::T)
 k_product_small(const float* __restrict__ p, float* __restrict__ u, const float2* __restrict__ tab2,
@@ -40,6 +46,7 @@ k_product_small(const float* __restrict__ p, float* __restrict__ u, const float2
   using Z = Small<LOGN>;
   using C = float2;
   constexpr int N = Z::N, M = 2 * N, R = 8, TR = Z::TR, TC = Z::TC;
+  if constexpr (Z::CTAS > 1) cluster_arrive();
   pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* const colb = reinterpret_cast<float4*>(smem_raw);            // [PC][N]: this block's columns
@@ -62,6 +69,7 @@ k_product_small(const float* __restrict__ p, float* __restrict__ u, const float2
 #pragma unroll
     for (int q = 0; q < R; ++q) sh[padi<3>(t + TR * q)] = v[q];
     GroupSync<TR, Z::GR>::sync(rl);
+    if constexpr (Z::CTAS > 1) cluster_wait();
     if (on) {
       const C wa = tw[2 * t], wb = tw[2 * t + 1];
       auto put = [&](int jp, float4 x) { cluster.map_shared_rank(colb, jp / Z::PC)[(jp % Z::PC) * N + row] = x; };
