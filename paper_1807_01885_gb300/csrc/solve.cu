@@ -203,7 +203,7 @@ __global__ void k_init_gap(const T* __restrict__ f, const T* __restrict__ p, T* 
 // and the set itself as bytes for the sweeps up to the update.
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T* __restrict__ p, T* __restrict__ g, const T* __restrict__ f, T* __restrict__ dp,
-                           const T* __restrict__ u, const uint8_t* __restrict__ cm, const uint8_t* __restrict__ xm,
+                           const T* __restrict__ u, uint8_t* __restrict__ cm, const uint8_t* __restrict__ xm,
                            double* partials, unsigned int* ticket, SolveState* st, size_t n) {
   pdl_enter();
   if (st->done) return;
@@ -249,6 +249,9 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T
       }
     }
     if (!any) continue;
+    // a scale below one may have taken subnormal pressures (a warm start's) to zero: those
+    // cells leave the set that the rest of the iteration reads
+    if (s1 < (T)0) stm4(cm, i4, pv);
     T sg[4], suu[4], sp[4], sc[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -1026,7 +1029,7 @@ void pk_chunk_launches(bem_kernel_s* k, cudaStream_t s) {
   for (int it = 0; it < CHUNK; ++it) {
     uint8_t *cm = m.cm[it & 1], *other = m.cm[1 - (it & 1)];   // this iteration's set; the previous, then the next one
     launch_matvec<T>(k, v.x, v.u, s, &st->mv_p_on);
-    launch_pdl(k_pk_begin<T>, c.rb, NTHREADS, 0, s, v.p, v.g, (const T*)v.f, v.x, (const T*)v.u, (const uint8_t*)cm,
+    launch_pdl(k_pk_begin<T>, c.rb, NTHREADS, 0, s, v.p, v.g, (const T*)v.f, v.x, (const T*)v.u, cm,
                (const uint8_t*)m.xm, part, tk, st, c.n);
     launch_pdl(k_pk_dir<T>, c.eb, NTHREADS, 0, s, (const uint8_t*)cm, (const uint8_t*)other, (const T*)v.g, v.t,
                (const SolveState*)st, c.n);
