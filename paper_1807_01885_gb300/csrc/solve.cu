@@ -616,23 +616,21 @@ __global__ void k_lin_alpha(const T* __restrict__ s, const T* __restrict__ q, co
   if constexpr (sizeof(T) == 4) {
     VEC_LOOP(i4, n) {
       bool in[4];
-      T sv[4], qv[4], p4[4];
+      T sv[4], qv[4], rv[4] = {(T)0, (T)0, (T)0, (T)0};
       if (!ldm4(C, i4, in)) continue;
       ld4(s, i4, sv);
       ld4(q, i4, qv);
+      if (force) ld4(r, i4, rv);
+      // term by term: K s and r add up to sums far below their terms, whose rounding a
+      // plain sum of four would leave in the means that are to remove it
 #pragma unroll
-      for (int e = 0; e < 4; ++e) p4[e] = in[e] ? sv[e] * qv[e] : (T)0;
-      a.add4(p4);
-      if (force) {
-        T rv[4];
-        ld4(r, i4, rv);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          qv[e] = in[e] ? qv[e] : (T)0;
-          rv[e] = in[e] ? rv[e] : (T)0;
+      for (int e = 0; e < 4; ++e) {
+        if (!in[e]) continue;
+        a.add(sv[e] * qv[e]);
+        if (force) {
+          aq.add(qv[e]);
+          ar.add(rv[e]);
         }
-        aq.add4(qv);
-        ar.add4(rv);
       }
     }
   } else {
@@ -670,7 +668,7 @@ __global__ void k_lin_update(T* __restrict__ x, T* __restrict__ r, const T* __re
   if constexpr (sizeof(T) == 4) {
     VEC_LOOP(i4, n) {
       bool in[4];
-      T xv[4], rv[4], sv[4], qv[4], r2[4];
+      T xv[4], rv[4], sv[4], qv[4];
       if (!ldm4(C, i4, in)) continue;
       ld4(x, i4, xv);
       ld4(r, i4, rv);
@@ -678,15 +676,13 @@ __global__ void k_lin_update(T* __restrict__ x, T* __restrict__ r, const T* __re
       ld4(q, i4, qv);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        if (in[e]) {
-          xv[e] += alpha * sv[e];
-          rv[e] = (rv[e] - rbar) - alpha * (qv[e] - qbar);
-        }
-        r2[e] = in[e] ? rv[e] * rv[e] : (T)0;
+        if (!in[e]) continue;
+        xv[e] += alpha * sv[e];
+        rv[e] = (rv[e] - rbar) - alpha * (qv[e] - qbar);
+        arr.add(rv[e] * rv[e]);
       }
       st4(x, i4, xv);
       st4(r, i4, rv);
-      arr.add4(r2);
     }
   } else {
     GRID_STRIDE(i, n) {
