@@ -332,8 +332,8 @@ k_layer_inf(const uint2* __restrict__ V, const bf16* __restrict__ Ww, const bf16
           }
           const float2 qb = sqb[j * 4 + t], qw = sqw[j * 4 + t];
           float h0 = acc[0] + qb.x, h1 = acc[1] + qb.y, h2 = acc[2] + qb.x, h3 = acc[3] + qb.y;
-          gelu2(h0, h1);
-          gelu2(h2, h3);
+          gelu2_proj(h0, h1);
+          gelu2_proj(h2, h3);
           sa += qw.x * h0 + qw.y * h1;
           sb2 += qw.x * h2 + qw.y * h3;
         }
