@@ -9,12 +9,16 @@
 //
 // A warp takes 16 pixels at a time and keeps hidden units as rows and pixels as columns:
 //   a (H x 16)  = Q1 (rows of weights as stored) x v (split hi/lo),
-//   dQ1 (H x W) = da (split; the accumulator layout is the operand layout) x v^T,
+//   dQ1 (H x W) = da (the accumulator layout is the operand layout) x v^T, both in three
+//                 parts (24 bits; six products of parts),
 //   dv (W x 16) = Q1^T x da.
 // v is loaded once in the order of the second product; the first and third need 8 x 8
 // blocks transposed, which movmatrix does on the packed bf16 parts.  dQ1 stays in
 // registers over all of a warp's tiles (each tile's product is added in float, since the
-// unit's accumulators truncate).
+// unit's accumulators truncate).  With two parts (16 bits) the products' rounding showed in
+// dQ1 on small grids, where the sum is short and its terms cancel: error up to 1.17 times
+// that of float products at 64 x 64 pixels (geometric mean of 36 networks of up to 16384
+// pixels 1.03; with three parts 1.007, gradient pass of 16 x 256 x 256 2.72 -> 2.75 ms).
 // Measured (GB300, 16 samples of 256 x 256, W = 32, H = 64): this kernel 218 us;
 // the gradient pass 3.10 -> 2.52 ms against the separate kernels (two layers forward,
 // gelu', two data and two weight gradients).
@@ -24,6 +28,14 @@ __device__ __forceinline__ unsigned trans8(unsigned x) {   // 8 x 8 b16 block, r
   unsigned d;
   asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(x));
   return d;
+}
+
+// x = hi + lo + m in three bf16 parts (24 bits), pairs packed
+__device__ __forceinline__ void split3(float x0, float x1, unsigned& hi, unsigned& lo, unsigned& m) {
+  split2(x0, x1, hi, lo);
+  const float r0 = (x0 - __uint_as_float(hi << 16)) - __uint_as_float(lo << 16);
+  const float r1 = (x1 - __uint_as_float(hi & 0xffff0000u)) - __uint_as_float(lo & 0xffff0000u);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r1), "f"(r0));
 }
 
 template <int KT, int MH>
@@ -36,6 +48,7 @@ k_proj_bwd(const float* __restrict__ V, const float* __restrict__ dout, const bf
   __shared__ float red[4][16 * MH * 16 * KT];
   __shared__ float red2[4][2][16 * MH];
   __shared__ float redb[4];
+  __shared__ float2 sqw[16 * MH];   // (q1, Q2) of hidden unit j
   const int lane = threadIdx.x % 32, g = lane / 4, t = lane % 4, wid = threadIdx.x / 32;
   // operand fragments of Q1 (rows j, k = c) and Q1^T (rows c, k = j)
   auto bits = [&](int j, int c) -> unsigned {
@@ -53,23 +66,16 @@ k_proj_bwd(const float* __restrict__ V, const float* __restrict__ dout, const bf
     sQ[mt][kb][lane] = make_uint4(a[0], a[1], a[2], a[3]);
     sQT[mt][kb][lane] = make_uint4(b[0], b[1], b[2], b[3]);
   }
+  for (int j = threadIdx.x; j < 16 * MH; j += 128)
+    sqw[j] = j < H ? make_float2(b2f(q1[j]), b2f(Q2[j])) : make_float2(0.f, 0.f);
   __syncthreads();
-  float qb[MH][2], qw[MH][2];
-#pragma unroll
-  for (int mt = 0; mt < MH; ++mt)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = 16 * mt + 8 * h + g;
-      qb[mt][h] = j < H ? b2f(q1[j]) : 0.f;
-      qw[mt][h] = j < H ? b2f(Q2[j]) : 0.f;
-    }
   float dq1[MH][NT][4] = {}, gq1[MH][2] = {}, gq2[MH][2] = {}, gb2 = 0.f;
   for (unsigned tile = blockIdx.x * 4 + wid; tile < tiles; tile += gridDim.x * 4) {
     const unsigned b = tile / tiles_per_sample, p0 = (tile - b * tiles_per_sample) * 16;
     const float* vb = V + (size_t)b * W * P;
     float* db = dV + (size_t)b * W * P;
-    // v: packed pairs of pixels 2t, 2t + 1 of rows c = 8 nt + g, hi and lo
-    unsigned vh[NT][2], vl[NT][2];
+    // v: packed pairs of pixels 2t, 2t + 1 of rows c = 8 nt + g, in three parts
+    unsigned vh[NT][2], vl[NT][2], vm[NT][2];
     float2 go[2];
 #pragma unroll
     for (int pt = 0; pt < 2; ++pt) {
@@ -81,7 +87,7 @@ k_proj_bwd(const float* __restrict__ V, const float* __restrict__ dout, const bf
         const int c = 8 * nt + g;
         const float2 x = (c < W && p < P) ? *reinterpret_cast<const float2*>(vb + (unsigned)c * P + p)
                                           : make_float2(0.f, 0.f);
-        split2(x.x, x.y, vh[nt][pt], vl[nt][pt]);
+        split3(x.x, x.y, vh[nt][pt], vl[nt][pt], vm[nt][pt]);
       }
     }
     unsigned th[NT][2], tl[NT][2];   // the same transposed: pixel rows, channel pairs
@@ -95,7 +101,7 @@ k_proj_bwd(const float* __restrict__ V, const float* __restrict__ dout, const bf
     float dv[KT][2][4] = {};
 #pragma unroll
     for (int mt = 0; mt < MH; ++mt) {
-      unsigned ah[4], al[4];   // da of rows 16 mt + g (+ 8), pixels 2t, 2t + 1 (+ 8): e = row half + 2 pt
+      unsigned ah[4], al[4], am[4];   // da of rows 16 mt + g (+ 8), pixels 2t, 2t + 1 (+ 8): e = row half + 2 pt
 #pragma unroll
       for (int pt = 0; pt < 2; ++pt) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -108,18 +114,22 @@ k_proj_bwd(const float* __restrict__ V, const float* __restrict__ dout, const bf
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+          const float2 q = sqw[16 * mt + 8 * h + g];
           float h0, h1, d0, d1;
-          gelu_both2(acc[2 * h] + qb[mt][h], acc[2 * h + 1] + qb[mt][h], h0, h1, d0, d1);
+          gelu_both2(acc[2 * h] + q.x, acc[2 * h + 1] + q.x, h0, h1, d0, d1);
           gq2[mt][h] += go[pt].x * h0 + go[pt].y * h1;
-          d0 *= go[pt].x * qw[mt][h];
-          d1 *= go[pt].y * qw[mt][h];
+          d0 *= go[pt].x * q.y;
+          d1 *= go[pt].y * q.y;
           gq1[mt][h] += d0 + d1;
-          split2(d0, d1, ah[h + 2 * pt], al[h + 2 * pt]);
+          split3(d0, d1, ah[h + 2 * pt], al[h + 2 * pt], am[h + 2 * pt]);
         }
       }
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         float d[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(d, ah, vm[nt][0], vm[nt][1]);
+        mma_bf16(d, am, vh[nt][0], vh[nt][1]);
+        mma_bf16(d, al, vl[nt][0], vl[nt][1]);
         mma_bf16(d, ah, vl[nt][0], vl[nt][1]);
         mma_bf16(d, al, vh[nt][0], vh[nt][1]);
         mma_bf16(d, ah, vh[nt][0], vh[nt][1]);
