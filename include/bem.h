@@ -218,8 +218,10 @@ bem_status bem_profile_passes(bem_kernel k, const void* p, void* u, int32_t reps
  * bem_set_radix rebuilds the stage twiddle tables on cuda_stream and drops the
  * handle's captured CG-iteration graph (the next solve on a capturable stream
  * captures it again).  The float path accepts 3 or 4 for each; the double path only
- * 3.  Other values give BEM_EINVAL; N < 16 ignores the call.  Synchronises the
- * stream. */
+ * 3.  Other values give BEM_EINVAL; N < 16 ignores the call.  bem_matvec in float at
+ * 16 <= N <= 64 is one launch of radix 8 whatever the choice, which then holds for the
+ * solves' passes; in double it has its own transforms (see bem_matvec).  Synchronises
+ * the stream. */
 bem_status bem_set_radix(bem_kernel k, int32_t row_log2_radix, int32_t col_log2_radix, void* cuda_stream);
 
 /* Autotuner of those choices: times every allowed radix of the row passes (forward

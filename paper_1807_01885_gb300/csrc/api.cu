@@ -452,12 +452,14 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
   if ((e = alloc_guarded(w, &w.table64, (size_t)(k->N + 1) * (k->N + 1) * sizeof(double))) != cudaSuccess)
     return fail(e, "cudaMalloc(table64)");
   if ((e = alloc_guarded(w, &w.tw, (size_t)k->M * 2 * k->elem)) != cudaSuccess) return fail(e, "cudaMalloc(tw)");
-  if ((e = alloc_guarded(w, &w.twr, (size_t)stage_tw_count(k->logN) * 2 * k->elem)) != cudaSuccess)
+  // twr, twpc: a second table of radix 8 behind the chosen radix's where the one-launch product needs it
+  const size_t tables = small_product_ok(k) ? 2 : 1;
+  if ((e = alloc_guarded(w, &w.twr, tables * stage_tw_count(k->logN) * 2 * k->elem)) != cudaSuccess)
     return fail(e, "cudaMalloc(twr)");
   if ((e = alloc_guarded(w, &w.twc, (size_t)stage_tw_count(k->logN + 1) * 2 * k->elem)) != cudaSuccess)
     return fail(e, "cudaMalloc(twc)");
   if (k->prec == BEM_FP32 &&
-      (e = alloc_guarded(w, &w.twpc, (size_t)pair_tw_count(k->logN + 1) * 4 * sizeof(float))) != cudaSuccess)
+      (e = alloc_guarded(w, &w.twpc, tables * pair_tw_count(k->logN + 1) * 4 * sizeof(float))) != cudaSuccess)
     return fail(e, "cudaMalloc(twpc)");
   if (k->prec == BEM_FP64 && k->logN >= 4) {
     if ((e = alloc_guarded(w, &w.fexp, (size_t)(2 * k->N + 1) * sizeof(int))) != cudaSuccess)

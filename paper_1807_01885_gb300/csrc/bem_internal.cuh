@@ -134,9 +134,9 @@ struct Workspace {
   void* table = nullptr;     // K^/M^2 in the path precision: N >= 16 (N+1) rows of N+4 (row j = column j), else blocked
   double* table64 = nullptr; // (N+1)^2 doubles, unscaled, row-major
   void* tw = nullptr;        // M complex: e^{-2 pi i k / M}
-  void* twr = nullptr;       // stage twiddles of the length-N register FFT (rows)
+  void* twr = nullptr;       // stage twiddles of the length-N register FFT (rows); see small_twr
   void* twc = nullptr;       // stage twiddles of the length-2N register FFT (columns)
-  void* twpc = nullptr;      // float path: broadcast stage twiddles of the paired column FFT (4N float4)
+  void* twpc = nullptr;      // float path: broadcast stage twiddles of the paired column FFT (4N float4); see small_twp
   int* fexp = nullptr;       // fixed-point product (double, N >= 16): exponents of the rows and columns (2N + 1)
   void* twf = nullptr;       // and its twiddles: M records, then the stages of lengths N and 2N
   void* vec = nullptr;       // solver vectors: p, g, t, r, u, f, x (N*N each)
@@ -285,8 +285,21 @@ template <typename T>
 void reg_twiddles(const bem_kernel_s* k, cudaStream_t s);
 template <typename T>
 void reg_prepare(const bem_kernel_s* k);
-// matvec_f32.cu: bem_matvec's product in one launch where the grid is small
-bool small_product_ok(const bem_kernel_s* k);
+// matvec.cu: stage twiddles of one FFT of length 2^logl (upper bound)
+int stage_tw_count(int logl);
+// float4 records of the paired FFT's stage twiddles for length 2^logl (upper bound)
+int pair_tw_count(int logl);
+// matvec_f32.cu: bem_matvec's product in one launch where the grid is small (float, N = 16 to
+// 64).  Its plan has radix 8; where the passes of the handle were given another radix, its
+// stage twiddles lie behind theirs in twr and twpc (bem_matvec would otherwise fall back to
+// three launches, 11.6 against 6.9 us a call, when bem_autotune picks radix 16 for solves).
+inline bool small_product_ok(const bem_kernel_s* k) { return k->prec == BEM_FP32 && k->logN >= 4 && k->logN <= 6; }
+inline float2* small_twr(const bem_kernel_s* k) {
+  return (float2*)k->ws.twr + (k->row_radix_alt ? 0 : stage_tw_count(k->logN));
+}
+inline float4* small_twp(const bem_kernel_s* k) {
+  return (float4*)k->ws.twpc + (k->col_radix_alt ? 0 : pair_tw_count(k->logN + 1));
+}
 void small_product(const bem_kernel_s* k, const float* p, float* u, cudaStream_t s);
 // matvec_fix.cu (double, N >= 16): one pass of the fixed-point product, its twiddles
 void fix_pass(const bem_kernel_s* k, int which, const double* p, double* u, cudaStream_t s);
@@ -299,9 +312,6 @@ void launch_product(const bem_kernel_s* k, const T* p, T* u, cudaStream_t s);
 // (what the first plain launch would set), so that a graph capture can follow
 template <typename T>
 void prepare_passes(const bem_kernel_s* k);
-int stage_tw_count(int logl);
-// float4 records of the paired FFT's stage twiddles for length 2^logl (upper bound)
-int pair_tw_count(int logl);
 size_t table_bytes(const bem_kernel_s* k);
 
 // solve.cu

@@ -7,10 +7,6 @@ template void reg_pass<float>(const bem_kernel_s*, int, const float*, float*, cu
 template void reg_twiddles<float>(const bem_kernel_s*, cudaStream_t);
 template void reg_prepare<float>(const bem_kernel_s*);
 
-bool small_product_ok(const bem_kernel_s* k) {
-  return k->prec == BEM_FP32 && k->logN >= kSmallMinLog && k->logN <= kSmallMaxLog && k->row_radix_alt &&
-         k->col_radix_alt;
-}
 void small_product(const bem_kernel_s* k, const float* p, float* u, cudaStream_t s) {
   small_logn(k->logN, [&](auto f) { f.run(k, p, u, s); });
 }

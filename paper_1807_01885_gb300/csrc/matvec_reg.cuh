@@ -508,10 +508,17 @@ void reg_prepare(const bem_kernel_s* k) {
 template <typename T>
 void reg_twiddles(const bem_kernel_s* k, cudaStream_t s) {
   k_stage_twiddles<T><<<64, 256, 0, s>>>((cplx<T>*)k->ws.twr, k->logN, row_logr<T>(k));
-  if constexpr (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4) {
     k_stage_twiddles_pair<<<64, 256, 0, s>>>((float4*)k->ws.twpc, k->logN + 1, col_logr<T>(k));
-  else
+    // the one-launch product's, of radix 8 whatever the passes use
+    if (small_product_ok(k) && !(k->row_radix_alt && k->col_radix_alt)) {
+      k_stage_twiddles<T><<<64, 256, 0, s>>>(small_twr(k), k->logN, 3);
+      k_stage_twiddles_pair<<<64, 256, 0, s>>>(small_twp(k), k->logN + 1, 3);
+      note_launches(2);
+    }
+  } else {
     k_stage_twiddles<T><<<64, 256, 0, s>>>((cplx<T>*)k->ws.twc, k->logN + 1, col_logr<T>(k));
+  }
 }
 
 }  // namespace bem

@@ -19,8 +19,6 @@
 
 namespace bem {
 
-constexpr int kSmallMinLog = 4, kSmallMaxLog = 6;
-
 template <int LOGN>
 struct Small {
   static constexpr int CTAS = LOGN <= 5 ? 1 : 4;
@@ -166,7 +164,7 @@ struct SmallLaunch {
   static void run(const bem_kernel_s* k, const float* p, float* u, cudaStream_t s) {
     prepare();
     launch_pdl(k_product_small<LOGN>, Small<LOGN>::CTAS, Small<LOGN>::T, Small<LOGN>::SMEM, s, p, u, (const float2*)k->ws.table,
-               (const float2*)k->ws.twr, (const float4*)k->ws.twpc, (const float2*)k->ws.tw);
+               (const float2*)small_twr(k), (const float4*)small_twp(k), (const float2*)k->ws.tw);
   }
 };
 
