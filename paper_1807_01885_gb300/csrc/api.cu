@@ -451,7 +451,16 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
   if ((e = alloc_guarded(w, &w.table, table_bytes(k))) != cudaSuccess) return fail(e, "cudaMalloc(table)");
   if ((e = alloc_guarded(w, &w.table64, (size_t)(k->N + 1) * (k->N + 1) * sizeof(double))) != cudaSuccess)
     return fail(e, "cudaMalloc(table64)");
-  if ((e = alloc_guarded(w, &w.tw, (size_t)k->M * 2 * k->elem)) != cudaSuccess) return fail(e, "cudaMalloc(tw)");
+  // tw; in double the fixed-point product's twiddles and exponents behind it (one allocation:
+  // each costs a new handle about 7 us)
+  const bool fix = k->prec == BEM_FP64 && k->logN >= 4;
+  const size_t tw_bytes = (size_t)k->M * 2 * k->elem, twf_bytes = fix ? fix_tw_bytes(k) : 0;
+  const size_t fexp_bytes = fix ? (size_t)(2 * k->N + 1) * sizeof(int) : 0;
+  if ((e = alloc_guarded(w, &w.tw, tw_bytes + twf_bytes + fexp_bytes)) != cudaSuccess) return fail(e, "cudaMalloc(tw)");
+  if (fix) {
+    w.twf = (char*)w.tw + tw_bytes;
+    w.fexp = (int*)((char*)w.twf + twf_bytes);
+  }
   // twr, twpc: a second table of radix 8 behind the chosen radix's where the one-launch product needs it
   const size_t tables = small_product_ok(k) ? 2 : 1;
   if ((e = alloc_guarded(w, &w.twr, tables * stage_tw_count(k->logN) * 2 * k->elem)) != cudaSuccess)
@@ -461,11 +470,6 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
   if (k->prec == BEM_FP32 &&
       (e = alloc_guarded(w, &w.twpc, tables * pair_tw_count(k->logN + 1) * 4 * sizeof(float))) != cudaSuccess)
     return fail(e, "cudaMalloc(twpc)");
-  if (k->prec == BEM_FP64 && k->logN >= 4) {
-    if ((e = alloc_guarded(w, &w.fexp, (size_t)(2 * k->N + 1) * sizeof(int))) != cudaSuccess)
-      return fail(e, "cudaMalloc(fexp)");
-    if ((e = alloc_guarded(w, &w.twf, fix_tw_bytes(k))) != cudaSuccess) return fail(e, "cudaMalloc(twf)");
-  }
   if ((e = alloc_guarded(w, &w.vec, 7 * n * k->elem)) != cudaSuccess) return fail(e, "cudaMalloc(vec)");
   if ((e = alloc_guarded(w, &w.mask, 2 * n + n / 4)) != cudaSuccess) return fail(e, "cudaMalloc(mask)");
   if ((e = alloc_guarded(w, &w.partials, 16 * 2048 * sizeof(double))) != cudaSuccess)
@@ -489,6 +493,7 @@ static bem_status make_kernel(const bem_kernel_desc* desc, int32_t n_layers, con
     delete k;
     return st;
   }
+  if (fix) fix_twiddles(k, s);
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "build_table");
   *out = k;
   return BEM_OK;

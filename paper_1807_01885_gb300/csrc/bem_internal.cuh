@@ -138,7 +138,7 @@ struct Workspace {
   void* twc = nullptr;       // stage twiddles of the length-2N register FFT (columns)
   void* twpc = nullptr;      // float path: broadcast stage twiddles of the paired column FFT (4N float4); see small_twp
   int* fexp = nullptr;       // fixed-point product (double, N >= 16): exponents of the rows and columns (2N + 1)
-  void* twf = nullptr;       // and its twiddles: M records, then the stages of lengths N and 2N
+  void* twf = nullptr;       // and its twiddles: M records, then the stages of lengths N and 2N (both inside tw's allocation)
   void* vec = nullptr;       // solver vectors: p, g, t, r, u, f, x (N*N each)
   uint8_t* mask = nullptr;   // N*N contact mask (adhesive), plus a second copy; PK: two contact sets, N*N/4 change flags
   double* partials = nullptr;// per-block partial sums

@@ -349,9 +349,16 @@ __device__ inline int4 fix_twiddle(int num, int den) {
   if (oct & 1) rn = den - rn;
   const DD pi4 = DD{0.78539816339744830962, 3.0616169978683829431e-17};
   const DD x = dd_mul(DD{(double)rn / (double)den, 0.0}, pi4), x2 = dd_mul(x, x);
-  DD c = DD{c_cos[11][0], c_cos[11][1]}, s = DD{c_sin[11][0], c_sin[11][1]};
+  // (the terms from x^12 / 12! on, 1e-10, in plain double)
+  double ch = c_cos[11][0], sh = c_sin[11][0];
+#pragma unroll
+  for (int k = 10; k >= 6; --k) {
+    ch = fma(ch, x2.h, c_cos[k][0]);
+    sh = fma(sh, x2.h, c_sin[k][0]);
+  }
+  DD c = DD{ch, 0.0}, s = DD{sh, 0.0};
 #pragma unroll 1
-  for (int k = 10; k >= 0; --k) {
+  for (int k = 5; k >= 0; --k) {
     c = dd_add(dd_mul(c, x2), DD{c_cos[k][0], c_cos[k][1]});
     s = dd_add(dd_mul(s, x2), DD{c_sin[k][0], c_sin[k][1]});
   }

@@ -325,10 +325,7 @@ bem_status build_table(bem_kernel_s* k, cudaStream_t s) {
     if (k->logN >= 4) k_table_square<double><<<256, 256, 0, s>>>(k->ws.table64, (double*)k->ws.table, k->N, scale);
     else k_table_block<double><<<256, 256, 0, s>>>(k->ws.table64, (double*)k->ws.table, k->N, scale);
     k_twiddles<double><<<(k->M + 255) / 256, 256, 0, s>>>((double2*)k->ws.tw, k->M);
-    if (k->logN >= 4) {
-      reg_twiddles<double>(k, s);
-      fix_twiddles(k, s);
-    }
+    if (k->logN >= 4) reg_twiddles<double>(k, s);
   } else {
     if (k->logN >= 4) k_table_pair<<<256, 256, 0, s>>>(k->ws.table64, (float2*)k->ws.table, k->N, scale);
     else k_table_block<float><<<256, 256, 0, s>>>(k->ws.table64, (float*)k->ws.table, k->N, scale);

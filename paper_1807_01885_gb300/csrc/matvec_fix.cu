@@ -237,22 +237,31 @@ k_row_inv_x(const I2* __restrict__ spec, const int* __restrict__ fexp, double* _
     urow[t + TT * q] = nan ? make_double2(bad, bad) : make_double2(from_fix(v[q].x, E), from_fix(v[q].y, E));
 }
 
-// tw[j] = e^{-2 pi i j / M}, j < M
-__global__ void k_twiddles_fix(int4* __restrict__ tw, int M) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) tw[m] = fix_twiddle(m, M);
-}
-// stage tables of the length-2^logl transform of radix 8, from tw of length 2^logm >= it
-__global__ void k_stage_twiddles_fix(int4* __restrict__ out, const int4* __restrict__ tw, int logl, int logm) {
-  int off = 0, ns = 1;
-  const int nst = logl / 3 + (logl % 3 ? 1 : 0);
-  for (int s = 0; s < nst; ++s) {
+// All twiddles of a handle in one launch, one per thread (the Taylor sums are chains of FP64
+// operations, so blocks of one warp spread them over the SMs): tw[j] = e^{-2 pi i j / M},
+// j < M = 2N, then the stage tables of the lengths N and M, L - 8 records each.
+__global__ void __launch_bounds__(32) k_twiddles_fix(int4* __restrict__ tw, int4* __restrict__ twr, int4* __restrict__ twc,
+                                                     int logn) {
+  const int N = 1 << logn, M = 2 * N;
+  int i = blockIdx.x * 32 + threadIdx.x;
+  if (i < M) {
+    tw[i] = fix_twiddle(i, M);
+    return;
+  }
+  i -= M;
+  const bool rows = i < N - 8;
+  if (!rows) i -= N - 8;
+  if (i >= M - 8) return;
+  int4* out = (rows ? twr : twc) + i;
+  const int logl = rows ? logn : logn + 1;
+  int ns = 8, s = 1;   // stage s: planes r = 1 .. Q - 1 of ns records
+  for (;; ++s) {
     const int Q = s < logl / 3 ? 8 : 1 << (logl % 3);
-    if (s > 0) {
-      const int cnt = (Q - 1) * ns, step = (1 << logm) / (ns * Q);
-      for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
-        out[off + i] = tw[(i % ns) * (i / ns + 1) * step];
-      off += cnt;
+    if (i < (Q - 1) * ns) {
+      *out = fix_twiddle((i % ns) * (i / ns + 1), ns * Q);
+      return;
     }
+    i -= (Q - 1) * ns;
     ns *= Q;
   }
 }
@@ -310,12 +319,10 @@ size_t fix_tw_bytes(const bem_kernel_s* k) {
   return ((size_t)k->M + stage_tw_count(k->logN) + stage_tw_count(k->logN + 1)) * sizeof(int4);
 }
 
-// twiddles of the recombination and of the stages of both lengths
+// twiddles of the recombination and of the stages of both lengths: they depend on N only
 void fix_twiddles(const bem_kernel_s* k, cudaStream_t s) {
   int4 *tw = (int4*)k->ws.twf, *twr = tw + k->M, *twc = twr + stage_tw_count(k->logN);
-  fx::k_twiddles_fix<<<(k->M + 63) / 64, 64, 0, s>>>(tw, k->M);
-  fx::k_stage_twiddles_fix<<<16, 256, 0, s>>>(twr, tw, k->logN, k->logN + 1);
-  fx::k_stage_twiddles_fix<<<16, 256, 0, s>>>(twc, tw, k->logN + 1, k->logN + 1);
-  note_launches(3);
+  fx::k_twiddles_fix<<<(2 * k->M + k->N + 31) / 32, 32, 0, s>>>(tw, twr, twc, k->logN);
+  note_launches(1);
 }
 }  // namespace bem
