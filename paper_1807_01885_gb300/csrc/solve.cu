@@ -161,16 +161,39 @@ __global__ void k_init_scale(const T* __restrict__ f, const T* __restrict__ q, c
   }
 }
 
+// The iteration's sets at the start: the contact set {p > 0}, no previous one, and the
+// groups with pending changes x.  Formed where p and x are: a launch of its own cost every
+// solve 2 to 5 us (N = 4 force control 277 / 271 us, which is what it took without the sets).
+template <typename T>
+__device__ __forceinline__ void init_sets4(const T (&pv)[4], const T (&xv)[4], size_t i4, uint8_t* cm, uint8_t* cm_prev,
+                                           uint8_t* xm) {
+  stm4(cm, i4, pv);
+  reinterpret_cast<unsigned*>(cm_prev)[i4] = 0u;
+  xm[i4] = xv[0] != (T)0 || xv[1] != (T)0 || xv[2] != (T)0 || xv[3] != (T)0 ? 1 : 0;
+}
+
 template <typename T>
 __global__ void k_init_apply(const T* __restrict__ f, T* __restrict__ q, const T* __restrict__ u,
-                             T* __restrict__ p, T* __restrict__ g, const SolveState* st, size_t n) {
+                             T* __restrict__ p, T* __restrict__ g, uint8_t* __restrict__ cm,
+                             uint8_t* __restrict__ cm_prev, uint8_t* __restrict__ xm, const SolveState* st, size_t n) {
   const T s = (T)st->scale;
   const double d = st->d;
   const T dT = (T)d;
-  GRID_STRIDE(i, n) {
-    p[i] = s * q[i];
-    g[i] = s * u[i] + (f[i] - dT);
-    q[i] = (T)0;   // q's slot holds the pending pressure changes from here on
+  VEC_LOOP(i4, n) {
+    T fv[4], qv[4], uv[4], pv[4], gv[4];
+    const T zero[4] = {(T)0, (T)0, (T)0, (T)0};
+    ld4(f, i4, fv);
+    ld4(q, i4, qv);
+    ld4(u, i4, uv);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      pv[e] = s * qv[e];
+      gv[e] = s * uv[e] + (fv[e] - dT);
+    }
+    st4(p, i4, pv);
+    st4(g, i4, gv);
+    st4(q, i4, zero);   // q's slot holds the pending pressure changes from here on
+    init_sets4(pv, zero, i4, cm, cm_prev, xm);
   }
 }
 
@@ -178,6 +201,7 @@ __global__ void k_init_apply(const T* __restrict__ f, T* __restrict__ q, const T
 // so that the first correction gives g = K p + f - d.
 template <typename T>
 __global__ void k_init_gap(const T* __restrict__ f, const T* __restrict__ p, T* __restrict__ g, T* __restrict__ dp,
+                           uint8_t* __restrict__ cm, uint8_t* __restrict__ cm_prev, uint8_t* __restrict__ xm,
                            const SolveState* st, size_t n) {
   const T dT = (T)st->d;
   VEC_LOOP(i4, n) {
@@ -188,6 +212,7 @@ __global__ void k_init_gap(const T* __restrict__ f, const T* __restrict__ p, T* 
     for (int e = 0; e < 4; ++e) gv[e] = fv[e] - dT;
     st4(g, i4, gv);
     st4(dp, i4, pv);
+    init_sets4(pv, pv, i4, cm, cm_prev, xm);
   }
 }
 
@@ -932,20 +957,6 @@ PkSets pk_sets(const bem_kernel_s* k) {
   return PkSets{{k->ws.mask, k->ws.mask + n}, k->ws.mask + 2 * n};
 }
 
-// First contact set {p > 0}, no previous one, and the groups with pending changes
-template <typename T>
-__global__ void k_init_sets(const T* __restrict__ p, const T* __restrict__ x, uint8_t* __restrict__ cm,
-                            uint8_t* __restrict__ cm_prev, uint8_t* __restrict__ xm, size_t n) {
-  VEC_LOOP(i4, n) {
-    T pv[4], xv[4];
-    ld4(p, i4, pv);
-    ld4(x, i4, xv);
-    stm4(cm, i4, pv);
-    reinterpret_cast<unsigned*>(cm_prev)[i4] = 0u;
-    xm[i4] = xv[0] != (T)0 || xv[1] != (T)0 || xv[2] != (T)0 || xv[3] != (T)0 ? 1 : 0;
-  }
-}
-
 // Initial state and first iterate of the Polonsky-Keer solve (asynchronous on s).
 template <typename T>
 bem_status pk_setup(bem_kernel_s* k, const bem_problem* prob, const T* pinit, cudaStream_t s) {
@@ -957,6 +968,7 @@ bem_status pk_setup(bem_kernel_s* k, const bem_problem* prob, const T* pinit, cu
   unsigned int* tk = k->ws.ticket;
   const bool force = prob->control == BEM_CTRL_FORCE;
   const double delta2 = k->desc.delta * k->desc.delta;
+  const PkSets m = pk_sets(k);
 
   SolveState init{};
   init.d = force ? 0.0 : prob->target;
@@ -987,11 +999,11 @@ bem_status pk_setup(bem_kernel_s* k, const bem_problem* prob, const T* pinit, cu
   if (pinit != nullptr) {
     if (pinit != v.p) BEM_CUDA_TRY(cudaMemcpyAsync(v.p, pinit, c.n * sizeof(T), cudaMemcpyDeviceToDevice, s));
     k_init_clamp<T><<<c.rb, NTHREADS, 0, s>>>(v.p, part, tk, st, c.n);
-    k_init_gap<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.p, v.g, v.x, st, c.n);
+    k_init_gap<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.p, v.g, v.x, m.cm[0], m.cm[1], m.xm, st, c.n);
     note_launches(2);
   } else if (force) {
     k_fill<T><<<c.eb, NTHREADS, 0, s>>>(v.p, prob->target / (delta2 * (double)c.n), c.n);
-    k_init_gap<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.p, v.g, v.x, st, c.n);
+    k_init_gap<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.p, v.g, v.x, m.cm[0], m.cm[1], m.xm, st, c.n);
     note_launches(2);
   } else {
     k_init_q<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.x, prob->target, c.n);
@@ -999,12 +1011,9 @@ bem_status pk_setup(bem_kernel_s* k, const bem_problem* prob, const T* pinit, cu
     launch_matvec<T>(k, v.x, v.u, s, nullptr);
     k_init_scale<T><<<c.rb, NTHREADS, 0, s>>>(v.f, v.x, v.u, part, tk, st, c.n);
     note_launches(1);
-    k_init_apply<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.x, v.u, v.p, v.g, st, c.n);
+    k_init_apply<T><<<c.eb, NTHREADS, 0, s>>>(v.f, v.x, v.u, v.p, v.g, m.cm[0], m.cm[1], m.xm, st, c.n);
     note_launches(1);
   }
-  const PkSets m = pk_sets(k);
-  k_init_sets<T><<<c.eb, NTHREADS, 0, s>>>(v.p, v.x, m.cm[0], m.cm[1], m.xm, c.n);
-  note_launches(1);
   BEM_CUDA_TRY(cudaGetLastError());
   return BEM_OK;
 }
