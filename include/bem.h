@@ -74,9 +74,10 @@ enum { BEM_OP_PERIODIC = 0, BEM_OP_OPEN = 1 };        /* bem_kernel_desc.op_kind
  * products of order N + 1 (about 50 ms at N = 2048). */
 typedef struct {
   int32_t N;
-  int32_t precision;    /* BEM_FP64: everything in double.  BEM_FP32: FFTs and vectors
-                           in float; reductions, CG scalars and the detachment
-                           test in double. */
+  int32_t precision;    /* BEM_FP64: everything in double (bem_matvec: transforms in 64-bit
+                           fixed point, more exact than double ones).  BEM_FP32: FFTs
+                           and vectors in float; reductions, CG scalars and the
+                           detachment test in double. */
   int32_t dc_mode;
   int32_t op_kind;      /* BEM_OP_PERIODIC or BEM_OP_OPEN (earlier versions: reserved, 0) */
   double delta, h, E1, nu1, E2, nu2;
@@ -182,7 +183,10 @@ bem_status bem_check_guards(bem_kernel k, int64_t* bad_bytes, void* cuda_stream)
 bem_status bem_debug_poke_guard(bem_kernel k, int32_t i);
 
 /* u = K p (Eq. 1 evaluated by Eq. 11).  p and u: N*N, host or device.  Device
- * arguments: asynchronous on the stream.  Host arguments: returns after u is written. */
+ * arguments: asynchronous on the stream.  Host arguments: returns after u is written.
+ * In double (N >= 16) the transforms run in 64-bit fixed point with a scale per transform,
+ * in float at 16 <= N <= 64 the whole product is one launch; the products inside a solve
+ * are the floating-point passes, and agree with this one to rounding, not bit for bit. */
 bem_status bem_matvec(bem_kernel k, const void* p, void* u, void* cuda_stream);
 
 /* Solves one contact problem; writes the pressure to p_out (N*N, host or device)

@@ -1037,9 +1037,9 @@ __global__ void __launch_bounds__(128) k_proj_tc(const float* __restrict__ X, in
   }
 }
 
-// c_k / N^2, the weights of the gradient of the inverse transform, for the current N
 #include "fno_infer.cuh"
 
+// c_k / N^2, the weights of the gradient of the inverse transform, for the current N
 __global__ void k_cky_scaled(const float* __restrict__ c, float* __restrict__ cs, int m, float inv) {
   FOR_N(k, (size_t)m) cs[k] = c[k] * inv;
 }
@@ -1765,7 +1765,10 @@ bem_status forward(bem_fno_s* f, int B, int N, const float* x, bool train, cudaS
   return BEM_OK;
 }
 
-// the one-pass inference (fno_infer.cuh): whole 16-pixel tiles, at most 16 modes
+// the one-pass inference (fno_infer.cuh): whole 16-pixel tiles, rows that a block's four
+// warps hold, at most 16 modes (with 32 the rows' coefficients beside the staged tiles are
+// 57 KB and more of shared memory, past a static array's 48, and the transform's
+// accumulators twice the registers); other networks take the training forward's kernels
 bool infer_ok(const bem_fno_s* f, int N) {
   return fused_size(f, N) && proj_ok(f, N) && N % 16 == 0 && N <= kInfMaxN && f->d.modes <= 16;
 }

@@ -11,7 +11,7 @@
 // last layer goes straight through the projection, so per layer the activations are read
 // once and written once and the last ones never leave the SM.
 // Measured on GB300 (32 channels, 16 modes, 4 layers, one sample of N = 2048): forward 3.02
-// -> 1.85 ms; a layer 345 us (1.07 GB) where layer and transform took 520; three blocks of
+// -> 1.87 ms; a layer 338 us (1.07 GB) where layer and transform took 520; three blocks of
 // 168 registers per SM against four of 128 1.81 / 1.93 ms, two 1.88.
 #pragma once
 

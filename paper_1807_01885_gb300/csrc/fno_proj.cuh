@@ -19,8 +19,8 @@
 // dQ1 on small grids, where the sum is short and its terms cancel: error up to 1.17 times
 // that of float products at 64 x 64 pixels (geometric mean of 36 networks of up to 16384
 // pixels 1.03; with three parts 1.007, gradient pass of 16 x 256 x 256 2.72 -> 2.75 ms).
-// Measured (GB300, 16 samples of 256 x 256, W = 32, H = 64): this kernel 218 us;
-// the gradient pass 3.10 -> 2.52 ms against the separate kernels (two layers forward,
+// Measured (GB300, 16 samples of 256 x 256, W = 32, H = 64): this kernel 244 us (218 with
+// two parts); the gradient pass 3.10 -> 2.52 ms, with two parts, against the separate kernels (two layers forward,
 // gelu', two data and two weight gradients).
 constexpr int kProjBlocks = 304;   // two per SM; one partial of every gradient each
 

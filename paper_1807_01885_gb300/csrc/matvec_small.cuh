@@ -9,7 +9,7 @@
 // sums by context).  Solves keep the passes, which their captured and plain iterations
 // share bit for bit.  N = 128 stays with them: 11.0 us on eight SMs against 6.4.
 // Measured on GB300, three passes / one launch: calls back to back N = 32 11.6 / 6.7 us,
-// 64 11.6 / 6.9; a product in a chain on the device N = 16 4.7 / 4.4 us, 32 4.7 / 4.8,
+// 64 11.6 / 6.9; a product in a chain on the device N = 16 4.7 / 4.2 us, 32 4.7 / 4.8,
 // 64 5.9 / 6.5 (eight blocks 6.9, two 8.1, one 10.4).
 #pragma once
 

@@ -102,8 +102,6 @@ __device__ __forceinline__ void finish(SolveState* st, int status) {
 // ---------------------------------------------------------------------------
 // Polonsky-Keer CG kernels
 
-// Initial guess for depth control: q = max(d - f, 0) scaled by the energy-optimal
-// factor s = <q, d - f> / <q, K q>; the gap then follows from u = K q as s u + f - d.
 // The sweeps touch what an iteration changes.  The contact set is a few per cent of the
 // cells of a rough surface and a sixth of a sphere's or a punch's window; outside it p and
 // t are zero and stay so, and the pending changes x are zero but for a few cells.  The set
@@ -111,10 +109,12 @@ __device__ __forceinline__ void finish(SolveState* st, int status) {
 // the other of two buffers (the previous set tells where t must be cleared), and xm holds
 // one byte per group of four cells whose x may not be zero.  Groups of four cells without
 // a contact cell then cost their byte word (and, where the gap itself moves, the gap's
-// arrays): 340 -> 150 MB per iteration at N = 2048, and in double the arithmetic of the
-// sums, which bounds those sweeps.  The sums only lose zeros: results are unchanged.
-// Measured on GB300, full sweeps / this: sphere N = 64 double 5.04 / 4.53 ms, rough surface
-// N = 2048 float 21.6 / 20.5 ms; a batch of 32 uneven grids gained 3 to 9 %.
+// arrays): 227 -> 137 MB read from memory per iteration at N = 2048 (ncu, cold caches, 3.3 %
+// in contact), and in double the arithmetic of the sums, which bounds those sweeps.  The
+// sums only lose zeros: results are unchanged.  Measured on GB300, full sweeps / this: sphere
+// N = 64 double 5.24 / 4.82 ms, punch N = 256 double 8.20 / 7.56, a batch of 32 uneven float
+// grids 31.6 / 30.4, rough surface N = 2048 float 18.04 / 17.76 (the four sweeps of an
+// iteration 77 / 75 us: their tails and the gap's arrays bound them).
 template <typename T>
 __device__ __forceinline__ void stm4(uint8_t* m, size_t i4, const T (&pv)[4]) {
   reinterpret_cast<uchar4*>(m)[i4] =
@@ -131,6 +131,8 @@ __device__ __forceinline__ bool ldm4(const uint8_t* m, size_t i4, bool (&o)[4]) 
 }
 __device__ __forceinline__ bool anym4(const uint8_t* m, size_t i4) { return reinterpret_cast<const unsigned*>(m)[i4] != 0u; }
 
+// Initial guess for depth control: q = max(d - f, 0) scaled by the energy-optimal
+// factor s = <q, d - f> / <q, K q>; the gap then follows from u = K q as s u + f - d.
 template <typename T>
 __global__ void k_init_q(const T* __restrict__ f, T* __restrict__ q, double d, size_t n) {
   const T dT = (T)d;
@@ -220,12 +222,14 @@ __global__ void k_init_gap(const T* __restrict__ f, const T* __restrict__ p, T* 
 // After a change of the contact set (refresh): the updates moved p by -tau t plus a
 // sparse change dp (cells projected to 0 or re-activated since the last correction),
 // accumulated in x; with u = K dp the gap becomes g + u, which keeps g a recursively
-// updated residual; x counts as cleared (k_pk_update rewrites it from 0).  (When a replacement was scheduled, x holds the
-// whole of p and g = f - d, so this recomputes g = K p + f - d from scratch.)
+// updated residual; x counts as cleared (k_pk_update rewrites it from 0).  (When a
+// replacement was scheduled, x holds the whole of p and g = f - d, so this recomputes
+// g = K p + f - d from scratch.)
 // Without a refresh only a pending load rescale is applied, with x scaled along.
 // Either way with the scale s actually applied to p: g = s g' + (s - 1)(d - f), p *= s.
-// Then sums over the contact set Ic = {p > 0}: sum g, count, sum g^2, sum u^2, sum p,
-// and the set itself as bytes for the sweeps up to the update.
+// Then sums over the contact set Ic = {p > 0}: sum g, count, sum g^2, sum u^2, sum p.
+// The set comes as bytes from the last update (the first one from the start kernels) and
+// is written again only where the scale has emptied cells.
 template <typename T>
 __global__ void __launch_bounds__(NTHREADS, sizeof(T) == 4 ? 4 : 1) k_pk_begin(T* __restrict__ p, T* __restrict__ g, const T* __restrict__ f, T* __restrict__ dp,
                            const T* __restrict__ u, uint8_t* __restrict__ cm, const uint8_t* __restrict__ xm,
